@@ -49,9 +49,10 @@ struct BatchArgs {
     int n2;            // power of two >= n_pop
     double* P;         // per block: 2 x n_pop x 6
     uint64_t* keys;    // per block: n_pop x 6
-    Deferred* queue;   // MIXED, per block: qcap entries
+    Deferred* queue;   // MIXED and FP64, per block: qcap entries
     unsigned qcap;
-    double* term;      // MIXED, per block: n_pop x max_ep chi^2 terms (row per candidate)
+    double* term;      // MIXED and FP64, per block: n_pop x max_ep chi^2 terms (row per candidate)
+    Cand* cands;       // per block: n_pop decoded candidates of the population being evaluated
     unsigned* next;    // work counter
     double* best_theta;
     double* best_chi2;
@@ -206,12 +207,13 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
     const int n_isl = a.n_isl;
     uint64_t* keys = a.keys + (size_t)blockIdx.x * n_pop * n_par;
     DeferSink sink{};
-    if (MODE == SBLM_MIXED) {
+    if (MODE != SBLM_FP32) {
         sink.queue = a.queue + (size_t)blockIdx.x * a.qcap;
         sink.queue_count = &s_qcount;
         sink.queue_cap = a.qcap;
     }
-    double* const term_blk = MODE == SBLM_MIXED ? a.term + (size_t)blockIdx.x * n_pop * a.max_ep : nullptr;
+    double* const term_blk = MODE != SBLM_FP32 ? a.term + (size_t)blockIdx.x * n_pop * a.max_ep : nullptr;
+    Cand* const cand_blk = a.cands + (size_t)blockIdx.x * n_pop;
     const int m = n_pop * n_par;
     double* const Pi = a.P + (size_t)blockIdx.x * n_isl * 2 * m;  // island i: rows Pi + i 2m (two buffers)
     sblm_ea_state* const st_g = a.isl_state + (size_t)blockIdx.x * n_isl;
@@ -277,32 +279,36 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
                     s_qcount = 0;
                     if (n_isl > 1) s_state = st_g[isl];
                 }
+                decode_candidates<true>(Pc, a.b, 0, n_pop, n_pop, cand_blk, nullptr);
                 __syncthreads();
                 for (int base = 0; base < n_pop; base += per_pass) {
                     const int cand = base + group;
                     const bool valid = cand < n_pop;
-                    const Cand k = group_candidate<true>(Pc, a.b, cand, valid, G);
+                    const Cand k = cand_blk[min(cand, n_pop - 1)];
                     double* A_row =
                         (a.blend && valid) ? a.A_scr + ((size_t)blockIdx.x * n_pop + cand) * a.max_ep : nullptr;
-                    double* term_row = (MODE == SBLM_MIXED && valid) ? term_blk + (size_t)cand * a.max_ep : nullptr;
+                    double* term_row = (MODE != SBLM_FP32 && valid) ? term_blk + (size_t)cand * a.max_ep : nullptr;
                     double chi = eval_run<MODE, true, true>(k, valid, cand, e0, e1, seg, view, A_row, nullptr, sink,
                                                             term_row);
                     for (int off = G / 2; off > 0; off >>= 1) chi += __shfl_xor_sync(0xffffffffu, chi, off);
                     if (g == 0 && valid) s_chi[cand] = chi;
                 }
                 __syncthreads();
-                if constexpr (MODE == SBLM_MIXED) {
+                if constexpr (MODE != SBLM_FP32) {
                     // the block's queued epochs, in FP64 from the FP64 data, each term to its place
                     // in the candidate's term row; then each candidate's row summed in a fixed order
-                    const unsigned n = min(s_qcount, a.qcap);
-                    for (unsigned i = threadIdx.x; i < n; i += blockDim.x) {
-                        const Deferred q = sink.queue[i];
-                        const Cand k = candidate<true>(Pc, a.b, q.c);
-                        double* A_rq = a.blend ? a.A_scr + ((size_t)blockIdx.x * n_pop + q.c) * a.max_ep : nullptr;
-                        const int64_t ge = e_begin + q.e;
-                        term_blk[(size_t)q.c * a.max_ep + q.e] = resolve_fp64(
-                            q.z, q.why, &k, a.t[ge], a.flux[ge], 1.0 / a.sigma[ge], A_rq, nullptr, q.e, true);
-                    }
+                    resolve_queue(
+                        sink.queue, min(s_qcount, a.qcap), threadIdx.x >> 5, blockDim.x >> 5,
+                        [&](int cq) { return cand_blk[cq]; },
+                        [&](int, int e) {
+                            const int64_t ge = e_begin + e;
+                            return EpochData{a.t[ge], a.flux[ge], 1.0 / a.sigma[ge]};
+                        },
+                        [&](int cq, int e, double A, uint8_t flag, uint32_t why, double fe, double we) {
+                            double* A_rq = a.blend ? a.A_scr + ((size_t)blockIdx.x * n_pop + cq) * a.max_ep : nullptr;
+                            term_blk[(size_t)cq * a.max_ep + e] =
+                                store_resolved<MODE>(A, flag, why, fe, we, A_rq, nullptr, e);
+                        });
                     __syncthreads();
                     for (int base = 0; base < n_pop; base += per_pass) {
                         const int cand = base + group;
@@ -579,7 +585,7 @@ sblm_status prepare(const double* t, const double* flux, const double* sigma, co
     // caustic-crossing model defers many), within 2^26 entries (~3 GB) over all blocks; epochs past
     // this are re-solved in place, one divergent lane at a time, so the size is a speed choice only
     const unsigned qcap =
-        mode == SBLM_MIXED
+        mode != SBLM_FP32
             ? (unsigned)std::max<long>(4096, std::min<long>((long)c.n_pop * max_ep / 4, (1L << 26) / blocks))
             : 0;
     const int k_order = st.scratch(sizeof(int) * n_lc);
@@ -590,7 +596,8 @@ sblm_status prepare(const double* t, const double* flux, const double* sigma, co
     const int k_ie = st.scratch(n_isl > 1 ? sizeof(double) * SBLM_NPAR * (size_t)blocks * n_isl : 0);
     const int k_keys = st.scratch(sizeof(uint64_t) * (size_t)c.n_pop * SBLM_NPAR * blocks);
     const int k_q = st.scratch(deferred_entry_bytes() * (size_t)qcap * blocks);
-    const int k_term = st.scratch(mode == SBLM_MIXED ? sizeof(double) * (size_t)c.n_pop * max_ep * blocks : 0);
+    const int k_term = st.scratch(mode != SBLM_FP32 ? sizeof(double) * (size_t)c.n_pop * max_ep * blocks : 0);
+    const int k_cand = st.scratch(sizeof(Cand) * (size_t)c.n_pop * blocks);
     const int k_next = st.scratch(sizeof(unsigned));
     const int k_genes = st.scratch(sizeof(double) * SBLM_NPAR * (size_t)n_lc);
     const int k_A = st.scratch(blend ? sizeof(double) * (size_t)blocks * c.n_pop * max_ep : 0);
@@ -669,6 +676,7 @@ sblm_status prepare(const double* t, const double* flux, const double* sigma, co
     a.queue = static_cast<Deferred*>(st.scratch_ptr(k_q));
     a.qcap = qcap;
     a.term = static_cast<double*>(st.scratch_ptr(k_term));
+    a.cands = static_cast<Cand*>(st.scratch_ptr(k_cand));
     a.next = static_cast<unsigned*>(st.scratch_ptr(k_next));
     a.best_theta = static_cast<double*>(st.dev(*i_th));
     a.best_chi2 = static_cast<double*>(st.dev(*i_c));

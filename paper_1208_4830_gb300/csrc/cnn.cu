@@ -774,7 +774,7 @@ Gen carve_gen(Carver& c, int B, int precision, bool own_theta) {
     g.A = c.take<double>((size_t)B * kBins);
     g.y = c.take<float>((size_t)B * 6);
     g.grid = c.take<double>(kBins);
-    g.mixed = c.take<unsigned char>(precision == SBLM_MIXED ? mixed_scratch_bytes(B, kBins, false) : 0);
+    g.mixed = c.take<unsigned char>(mixed_scratch_bytes(precision, B, kBins, false));
     g.ctr = c.take<int64_t>(2);
     return g;
 }

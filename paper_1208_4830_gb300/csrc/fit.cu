@@ -108,10 +108,9 @@ extern "C" sblm_status sblm_fit(const double* t, const double* flux, const doubl
     const int k_keys = st.scratch(sizeof(uint64_t) * m);
     const int k_state = st.scratch(sizeof(sblm_ea_state));
     const int G = choose_group(n_pop, n_ep);
-    const bool mixed = params->precision == SBLM_MIXED;
-    const int k_mx = st.scratch(mixed ? mixed_scratch_bytes(n_pop, n_ep, true) : 0);
+    const int k_mx = st.scratch(mixed_scratch_bytes(params->precision, n_pop, n_ep, true));
     const PolishMixed pmx = polish_mixed_layout(n_ep);
-    const int k_pmx = st.scratch(mixed && polish_fev > 0 ? pmx.block_bytes : 0);
+    const int k_pmx = st.scratch(params->precision == SBLM_MIXED && polish_fev > 0 ? pmx.block_bytes : 0);
     SBLM_TRY(st.begin());
 
     double* P[2] = {static_cast<double*>(st.scratch_ptr(k_P0)), static_cast<double*>(st.scratch_ptr(k_P1))};

@@ -19,31 +19,42 @@ namespace {
 
 constexpr int kBlock = 256;
 
-// MIXED, second pass: the queued epochs in full warps over the whole GPU. Each chi^2 term goes to
-// its (candidate, epoch) place in the dense term array (no atomics), so the sums of the third pass
-// do not depend on the order in which the queue was filled.
-template <bool CHI2, bool FROM_GENES>
-__global__ void __launch_bounds__(256) resolve_kernel(const double* __restrict__ src, Bounds bounds,
-                                                      const double* __restrict__ t,
-                                                      const double* __restrict__ flux,
-                                                      const double* __restrict__ sigma, int n_ep,
-                                                      const Deferred* __restrict__ queue,
-                                                      const unsigned* __restrict__ count, unsigned cap,
-                                                      double* __restrict__ A_out, uint8_t* __restrict__ flags,
-                                                      double* __restrict__ term) {
-    const unsigned n = min(*count, cap);
-    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const Deferred q = queue[i];
-        const Cand k = candidate<FROM_GENES>(src, bounds, q.c);
-        const double fe = CHI2 ? flux[q.e] : 0.0;
-        const double we = CHI2 ? 1.0 / sigma[q.e] : 0.0;
-        const double tm = resolve_fp64(q.z, q.why, &k, t[q.e], fe, we, A_out ? A_out + (size_t)q.c * n_ep : nullptr,
-                                       flags ? flags + (size_t)q.c * n_ep : nullptr, q.e, CHI2);
-        if (CHI2) term[(size_t)q.c * n_ep + q.e] = tm;
-    }
+// bytes of the staged lightcurve, rounded up so that what follows it in shared memory is aligned
+__host__ __device__ constexpr size_t staged_span(int mode, bool chi2, int n_ep) {
+    return ((size_t)n_ep * (mode == SBLM_FP64 ? sizeof(double) * (chi2 ? 3 : 1) : sizeof(float4)) + 15) & ~size_t(15);
 }
 
-// MIXED, third pass: chi^2 of candidate (warp) c as the sum of its term row in a fixed order
+constexpr int kResolveBlock = 128;
+
+// MIXED and FP64, second pass: the queued epochs, six per warp (refine.cuh), over the whole GPU: the
+// first epochs of the queue go to one warp of every block, so that a short queue spreads over the SMs
+// (the FP64 pipe is the bound). Each chi^2 term goes to its (candidate, epoch) place in the dense term
+// array (no atomics), so the sums of the third pass do not depend on the order in which the queue was
+// filled.
+template <int MODE, bool CHI2>
+__global__ void __launch_bounds__(kResolveBlock) resolve_kernel(const Cand* __restrict__ cands,
+                                                                const double* __restrict__ t,
+                                                                const double* __restrict__ flux,
+                                                                const double* __restrict__ sigma, int n_ep,
+                                                                const Deferred* __restrict__ queue,
+                                                                const unsigned* __restrict__ count, unsigned cap,
+                                                                double* __restrict__ A_out, uint8_t* __restrict__ flags,
+                                                                double* __restrict__ term) {
+    const unsigned n = min(*count, cap);
+    resolve_queue(
+        queue, n, (threadIdx.x >> 5) * gridDim.x + blockIdx.x, gridDim.x * (kResolveBlock / 32),
+        [&](int c) { return cands[c]; },
+        [&](int, int e) {
+            return EpochData{t[e], CHI2 ? flux[e] : 0.0, CHI2 ? 1.0 / sigma[e] : 0.0};
+        },
+        [&](int c, int e, double A, uint8_t flag, uint32_t why, double fe, double we) {
+            const double tm = store_resolved<MODE>(A, flag, why, fe, we, A_out ? A_out + (size_t)c * n_ep : nullptr,
+                                                   flags ? flags + (size_t)c * n_ep : nullptr, e);
+            if (CHI2) term[(size_t)c * n_ep + e] = tm;
+        });
+}
+
+// MIXED and FP64, third pass: chi^2 of candidate (warp) c as the sum of its term row in a fixed order
 // (lane l adds epochs l, l + 32, ... in order, then a fixed butterfly)
 __global__ void term_sum_kernel(int n_cand, int n_ep, const double* __restrict__ term, double* __restrict__ chi2_out) {
     const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
@@ -95,12 +106,16 @@ __global__ void __launch_bounds__(kBlock, forward_min_blocks(MODE))
     forward_kernel(const double* __restrict__ src, Bounds bounds, int n_cand, const double* __restrict__ t,
                    const double* __restrict__ flux, const double* __restrict__ sigma, int n_ep,
                    double* __restrict__ A_out, uint8_t* __restrict__ flags, double* __restrict__ chi2_out, int G,
-                   DeferSink sink, double* __restrict__ term) {
+                   DeferSink sink, double* __restrict__ term, Cand* __restrict__ cands) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const LCView lc = STAGED ? stage_lightcurve<MODE, CHI2>(smem, t, flux, sigma, n_ep)
-                             : LCView{t, flux, sigma, nullptr, nullptr, nullptr, nullptr};
     const int group = threadIdx.x / G, g = threadIdx.x % G;
     const int per_block = blockDim.x / G;
+    Cand* s_cand = reinterpret_cast<Cand*>(smem + (STAGED ? staged_span(MODE, CHI2, n_ep) : 0));
+    decode_candidates<FROM_GENES>(src, bounds, blockIdx.x * per_block, per_block, n_cand, s_cand,
+                                  MODE != SBLM_FP32 ? cands : nullptr);
+    const LCView lc = STAGED ? stage_lightcurve<MODE, CHI2>(smem, t, flux, sigma, n_ep)
+                             : LCView{t, flux, sigma, nullptr, nullptr, nullptr, nullptr};
+    if (!STAGED) __syncthreads();
     const int c = blockIdx.x * per_block + group;
     const bool valid = c < n_cand;
     const int seg = (n_ep + G - 1) / G;
@@ -108,12 +123,12 @@ __global__ void __launch_bounds__(kBlock, forward_min_blocks(MODE))
     // + warp), so each warp samples the whole lightcurve and the warps carry similar work
     const int gs = G > 32 ? (g & 31) * (G >> 5) + (g >> 5) : g;
     const int e0 = min(n_ep, gs * seg), e1 = min(n_ep, e0 + seg);
-    const Cand k = group_candidate<FROM_GENES>(src, bounds, c, valid, G);
+    const Cand k = s_cand[group];
     double* A_row = (A_out && valid) ? A_out + (size_t)c * n_ep : nullptr;
     uint8_t* f_row = (flags && valid) ? flags + (size_t)c * n_ep : nullptr;
-    double* term_row = (MODE == SBLM_MIXED && CHI2 && valid) ? term + (size_t)c * n_ep : nullptr;
+    double* term_row = (MODE != SBLM_FP32 && CHI2 && valid) ? term + (size_t)c * n_ep : nullptr;
     double chi = eval_run<MODE, CHI2, STAGED>(k, valid, c, e0, e1, seg, lc, A_row, f_row, sink, term_row);
-    if (!CHI2 || MODE == SBLM_MIXED) return;  // MIXED: the term rows are summed after the re-solve
+    if (!CHI2 || MODE != SBLM_FP32) return;  // else the term rows are summed after the re-solve
     // deterministic reduction over the candidate's G threads
     const int width = min(G, 32);
     for (int off = width / 2; off > 0; off >>= 1) chi += __shfl_xor_sync(0xffffffffu, chi, off);
@@ -135,31 +150,37 @@ __global__ void __launch_bounds__(kBlock, forward_min_blocks(MODE))
 template <int MODE, bool CHI2, bool STAGED, bool FROM_GENES>
 cudaError_t launch_t(const ForwardArgs& a, cudaStream_t s) {
     auto kern = forward_kernel<MODE, CHI2, STAGED, FROM_GENES>;
-    const size_t smem = STAGED ? staged_bytes(MODE, CHI2, a.n_ep) : 0;
+    const int per_block = kBlock / a.G;
+    const size_t smem = (STAGED ? staged_span(MODE, CHI2, a.n_ep) : 0) + sizeof(Cand) * (size_t)per_block;
     // opt in to more than 48 KB (dynamic plus the kernel's static shared memory) once per
     // device and size
     cudaError_t e = raise_smem_limit((const void*)kern, smem);
     if (e != cudaSuccess) return e;
-    const int per_block = kBlock / a.G;
     const int grid = (a.n_cand + per_block - 1) / per_block;
     DeferSink sink{};
     MixedLayout ml;
     double* term = nullptr;
-    if (MODE == SBLM_MIXED) {
-        ml = mixed_layout(a.n_cand, a.n_ep, CHI2);
+    Cand* cands = nullptr;
+    if (MODE != SBLM_FP32) {
+        ml = mixed_layout(MODE, a.n_cand, a.n_ep, CHI2);
         char* m = static_cast<char*>(a.mixed);
         sink.queue = reinterpret_cast<Deferred*>(m);
         sink.queue_count = reinterpret_cast<unsigned*>(m + ml.off_count);
         sink.queue_cap = ml.queue_cap;
+        cands = reinterpret_cast<Cand*>(m + ml.off_cand);
         term = CHI2 ? reinterpret_cast<double*>(m + ml.off_term) : nullptr;
+        e = cudaMemsetAsync(sink.queue_count, 0, sizeof(unsigned), s);
+        if (e != cudaSuccess) return e;
     }
     kern<<<grid, kBlock, smem, s>>>(a.src, a.bounds, a.n_cand, a.t, a.flux, a.sigma, a.n_ep, a.A_out, a.flags,
-                                    a.chi2_out, a.G, sink, term);
+                                    a.chi2_out, a.G, sink, term, cands);
     e = cudaGetLastError();
-    if (e != cudaSuccess || MODE != SBLM_MIXED) return e;
-    const int rgrid = (int)std::min<unsigned>((ml.queue_cap + 255) / 256, 8u * (unsigned)device_sm_count());
-    resolve_kernel<CHI2, FROM_GENES><<<rgrid, 256, 0, s>>>(a.src, a.bounds, a.t, a.flux, a.sigma, a.n_ep, sink.queue,
-                                                          sink.queue_count, ml.queue_cap, a.A_out, a.flags, term);
+    if (e != cudaSuccess || MODE == SBLM_FP32) return e;
+    const unsigned per_rblock = kResolvePerWarp * (kResolveBlock / 32);
+    const int rgrid = (int)std::min<unsigned>((ml.queue_cap + per_rblock - 1) / per_rblock,
+                                              4u * (unsigned)device_sm_count());
+    resolve_kernel<MODE, CHI2><<<rgrid, kResolveBlock, 0, s>>>(cands, a.t, a.flux, a.sigma, a.n_ep, sink.queue,
+                                                               sink.queue_count, ml.queue_cap, a.A_out, a.flags, term);
     e = cudaGetLastError();
     if (e != cudaSuccess || !CHI2) return e;
     term_sum_kernel<<<(int)(((long)a.n_cand * 32 + 255) / 256), 256, 0, s>>>(a.n_cand, a.n_ep, term, a.chi2_out);
@@ -194,16 +215,31 @@ int choose_group(int n_cand, int n_ep) {
     return (int)std::max(1L, std::min(g, cap));
 }
 
-MixedLayout mixed_layout(int n_cand, int n_ep, bool chi2) {
+namespace {
+
+// FP64 runs in chunks of candidates of at most this many epochs, one after the other in the same
+// scratch (a chunk of this size fills the GPU for a millisecond and its term rows stay in L2)
+constexpr long kFp64ChunkEpochs = 1L << 22;
+
+int fp64_chunk(int n_cand, int n_ep) {
+    return (int)std::min<long>(n_cand, std::max<long>(1, kFp64ChunkEpochs / std::max(1, n_ep)));
+}
+
+}  // namespace
+
+MixedLayout mixed_layout(int mode, int n_cand, int n_ep, bool chi2) {
     MixedLayout l;
-    if (n_cand <= 0 || n_ep <= 0) return l;
-    // a queue entry for one epoch in 32 (0.55% of the sweep's epochs defer, 4.2% of those of the
-    // trajectories aimed at caustics), at least 4096 and at most 2^24 entries (0.9 GB)
+    if (mode == SBLM_FP32 || n_cand <= 0 || n_ep <= 0) return l;
+    if (mode == SBLM_FP64) n_cand = fp64_chunk(n_cand, n_ep);
+    // a queue entry for one epoch in 32 (0.35% of the sweep's epochs defer in MIXED, 2.6% of those of
+    // the trajectories aimed at caustics), for FP64's wider triggers one in 8; at least 4096 and at most
+    // 2^24 entries (0.9 GB)
     const long n = (long)n_cand * n_ep;
-    l.queue_cap = (unsigned)std::min<long>(std::max<long>(n / 32, 4096), 1L << 24);
+    l.queue_cap = (unsigned)std::min<long>(std::max<long>(n / (mode == SBLM_FP64 ? 8 : 32), 4096), 1L << 24);
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
     l.off_count = up(sizeof(Deferred) * (size_t)l.queue_cap);
-    l.off_term = up(l.off_count + sizeof(unsigned));
+    l.off_cand = up(l.off_count + sizeof(unsigned));
+    l.off_term = up(l.off_cand + sizeof(Cand) * (size_t)n_cand);
     l.bytes = up(l.off_term + (chi2 ? sizeof(double) * (size_t)n : 0));
     return l;
 }
@@ -212,18 +248,22 @@ size_t deferred_entry_bytes() { return sizeof(Deferred); }
 
 cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t s) {
     if (a.n_cand <= 0 || a.n_ep <= 0) return cudaSuccess;
-    if (a.mode == SBLM_MIXED) {
-        if (!a.mixed) return cudaErrorInvalidValue;
-        const MixedLayout ml = mixed_layout(a.n_cand, a.n_ep, a.chi2_out != nullptr);
-        cudaError_t e = cudaMemsetAsync(static_cast<char*>(a.mixed) + ml.off_count, 0, sizeof(unsigned), s);
+    if (a.mode != SBLM_FP32 && !a.mixed) return cudaErrorInvalidValue;
+    const bool chi2 = a.chi2_out != nullptr;
+    if (a.mode == SBLM_MIXED) return chi2 ? launch_m<SBLM_MIXED, true>(a, s) : launch_m<SBLM_MIXED, false>(a, s);
+    if (a.mode != SBLM_FP64) return chi2 ? launch_m<SBLM_FP32, true>(a, s) : launch_m<SBLM_FP32, false>(a, s);
+    const int chunk = fp64_chunk(a.n_cand, a.n_ep);
+    for (int c = 0; c < a.n_cand; c += chunk) {
+        ForwardArgs p = a;
+        p.src = a.src + (size_t)SBLM_NPAR * c;
+        p.n_cand = std::min(chunk, a.n_cand - c);
+        if (a.A_out) p.A_out = a.A_out + (size_t)c * a.n_ep;
+        if (a.flags) p.flags = a.flags + (size_t)c * a.n_ep;
+        if (chi2) p.chi2_out = a.chi2_out + c;
+        const cudaError_t e = chi2 ? launch_m<SBLM_FP64, true>(p, s) : launch_m<SBLM_FP64, false>(p, s);
         if (e != cudaSuccess) return e;
     }
-    const bool chi2 = a.chi2_out != nullptr;
-    switch (a.mode) {
-        case SBLM_FP64: return chi2 ? launch_m<SBLM_FP64, true>(a, s) : launch_m<SBLM_FP64, false>(a, s);
-        case SBLM_MIXED: return chi2 ? launch_m<SBLM_MIXED, true>(a, s) : launch_m<SBLM_MIXED, false>(a, s);
-        default: return chi2 ? launch_m<SBLM_FP32, true>(a, s) : launch_m<SBLM_FP32, false>(a, s);
-    }
+    return cudaSuccess;
 }
 
 sblm_status check_theta_host(const double* theta, int n_cand) {
@@ -265,7 +305,7 @@ extern "C" sblm_status sblm_magnification(const double* theta, int32_t n_cand, c
     SBLM_TRY(st.arg(A_out, sizeof(double) * (size_t)n_cand * n_ep, false, true, &i_A));
     SBLM_TRY(st.arg(flags, flags ? (size_t)n_cand * n_ep : 0, false, true, &i_f));
     const int G = choose_group(n_cand, n_ep);
-    const int k_mx = st.scratch(precision == SBLM_MIXED ? mixed_scratch_bytes(n_cand, n_ep, false) : 0);
+    const int k_mx = st.scratch(mixed_scratch_bytes(precision, n_cand, n_ep, false));
     bool on_dev = true;
     SBLM_TRY(is_device_pointer(theta, &on_dev));
     if (!on_dev) SBLM_TRY(check_theta_host(theta, n_cand));
@@ -307,7 +347,7 @@ static sblm_status chi2_impl(const double* src, bool genes, const Bounds& b, int
     SBLM_TRY(st.arg(sigma, sizeof(double) * (size_t)n_ep, true, false, &i_s));
     SBLM_TRY(st.arg(chi2_out, sizeof(double) * (size_t)n_cand, false, true, &i_c));
     const int G = choose_group(n_cand, n_ep);
-    const int k_mx = st.scratch(precision == SBLM_MIXED ? mixed_scratch_bytes(n_cand, n_ep, true) : 0);
+    const int k_mx = st.scratch(mixed_scratch_bytes(precision, n_cand, n_ep, true));
     bool on_dev = true;
     SBLM_TRY(is_device_pointer(src, &on_dev));
     if (!on_dev && !genes) SBLM_TRY(check_theta_host(src, n_cand));
@@ -367,7 +407,7 @@ extern "C" sblm_status sblm_chi2_blend(const double* theta, int32_t n_cand, cons
     SBLM_TRY(st.arg(f_out, f_out ? sizeof(double) * (size_t)n_cand : 0, false, true, &i_fo));
     const int G = choose_group(n_cand, n_ep);
     const int k_A = st.scratch(sizeof(double) * (size_t)n_cand * n_ep);
-    const int k_mx = st.scratch(precision == SBLM_MIXED ? mixed_scratch_bytes(n_cand, n_ep, false) : 0);
+    const int k_mx = st.scratch(mixed_scratch_bytes(precision, n_cand, n_ep, false));
     bool d = true;
     SBLM_TRY(is_device_pointer(theta, &d));
     if (!d) SBLM_TRY(check_theta_host(theta, n_cand));

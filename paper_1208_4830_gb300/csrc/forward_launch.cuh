@@ -34,21 +34,24 @@ struct ForwardArgs {
     double* chi2_out = nullptr;    // optional [n_cand]; null -> no chi^2
     int mode = SBLM_FP64;
     int G = 32;                    // threads per candidate (power of two, <= 256)
-    // MIXED only: mixed_scratch_bytes(n_cand, n_ep, chi2_out != null) bytes of device scratch
-    // (256-byte aligned) for the re-solve queue, its counter and the chi^2 terms; launch_forward
-    // zeroes the counter
+    // MIXED and FP64: mixed_scratch_bytes(mode, n_cand, n_ep, chi2_out != null) bytes of device
+    // scratch (256-byte aligned) for the re-solve queue, its counter, the decoded candidates and the
+    // chi^2 terms; launch_forward zeroes the counter
     void* mixed = nullptr;
 };
 
-// MIXED scratch of one forward pass: the re-solve queue (an entry for one epoch in 32; an epoch
-// that finds it full is re-solved in place), its counter and, when chi^2 is wanted, the dense
-// n_cand x n_ep array of chi^2 terms that is summed row by row in a fixed order
+// MIXED and FP64 scratch of one forward pass: the re-solve queue (an epoch that finds it full is
+// re-solved in place), its counter, the decoded candidates and, when chi^2 is wanted, the dense
+// n_cand x n_ep array of chi^2 terms that is summed row by row in a fixed order. FP64 passes its
+// candidates through one chunk's scratch. FP32 needs none (0 bytes).
 struct MixedLayout {
     unsigned queue_cap = 0;
-    size_t off_count = 0, off_term = 0, bytes = 0;
+    size_t off_count = 0, off_cand = 0, off_term = 0, bytes = 0;
 };
-MixedLayout mixed_layout(int n_cand, int n_ep, bool chi2);
-inline size_t mixed_scratch_bytes(int n_cand, int n_ep, bool chi2) { return mixed_layout(n_cand, n_ep, chi2).bytes; }
+MixedLayout mixed_layout(int mode, int n_cand, int n_ep, bool chi2);
+inline size_t mixed_scratch_bytes(int mode, int n_cand, int n_ep, bool chi2) {
+    return mixed_layout(mode, n_cand, n_ep, chi2).bytes;
+}
 size_t deferred_entry_bytes();
 
 size_t staged_bytes(int mode, bool chi2, int n_ep);

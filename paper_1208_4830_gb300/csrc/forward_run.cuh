@@ -4,6 +4,7 @@
 
 #include "forward.cuh"
 #include "forward_launch.cuh"
+#include "refine.cuh"
 
 namespace sblm {
 
@@ -72,54 +73,57 @@ __device__ __forceinline__ Cand candidate(const double* __restrict__ src, const 
     return k;
 }
 
-// The candidate of a group of G threads (G a power of two; groups are aligned to G within the
-// warp, or span whole warps when G > 32), decoded once per warp-part by its first lane and
-// broadcast by shuffles: the decode's FP64 exp10, sincos and division run on the slow FP64 pipe.
-// Every lane of the warp must call it.
+// Decode the block's candidates c0 .. c0 + n - 1 (those below n_cand) into shared memory, one thread
+// each, and into `out` (when given) for the re-solve; the caller's next barrier publishes them. The
+// decode's exp10, sincos and division are about 120 instructions of the FP64 pipe, which takes them
+// at the same rate from a warp with one active lane as from a full one, so a block's candidates
+// share one or a few warps instead of every warp decoding its own.
 template <bool FROM_GENES>
-__device__ __forceinline__ Cand group_candidate(const double* __restrict__ src, const Bounds& b, int c, bool valid,
-                                                int G) {
-    const int lane = threadIdx.x & 31;
-    const int src_lane = G < 32 ? (lane & ~(G - 1)) : 0;
-    Cand k{};
-    if (lane == src_lane && valid) k = candidate<FROM_GENES>(src, b, c);
-    k.t0 = __shfl_sync(0xffffffffu, k.t0, src_lane);
-    k.inv_tE = __shfl_sync(0xffffffffu, k.inv_tE, src_lane);
-    k.u0 = __shfl_sync(0xffffffffu, k.u0, src_lane);
-    k.sa = __shfl_sync(0xffffffffu, k.sa, src_lane);
-    k.ca = __shfl_sync(0xffffffffu, k.ca, src_lane);
-    k.d = __shfl_sync(0xffffffffu, k.d, src_lane);
-    k.q = __shfl_sync(0xffffffffu, k.q, src_lane);
-    return k;
+__device__ __forceinline__ void decode_candidates(const double* __restrict__ src, const Bounds& b, int c0, int n,
+                                                  int n_cand, Cand* s_cand, Cand* out) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        Cand k{};
+        if (c0 + i < n_cand) {
+            k = candidate<FROM_GENES>(src, b, c0 + i);
+            if (out) out[c0 + i] = k;
+        }
+        s_cand[i] = k;
+    }
 }
 
-// the MIXED re-solve's Aberth stop rule (relative correction), see solve_epoch
+// the general re-solve's Aberth stop rule (relative correction), see solve_epoch
 constexpr double kResolveCubic = 1e-6;
 
-// FP64 re-solve of one deferred epoch (MIXED), warm-started from its FP32 roots; returns the
-// chi^2 term from the FP64 flux fe and weight we = 1/sigma. Out of line: an FP32 lane that must
-// do it in place keeps its state on the stack instead of competing with the FP64 solver for
-// registers.
-static __device__ __noinline__ double resolve_fp64(const cx<float>* z32, uint32_t why, const Cand* kk,
-                                                   double te, double fe, double we, double* A_row,
-                                                   uint8_t* f_row, int e, bool chi2) {
+// General FP64 solve of one epoch, warm-started from its FP32 roots: what resolve_group leaves open.
+// Out of line: a lane that must do it in place keeps its state on the stack instead of competing
+// with the FP64 solver for registers.
+static __device__ __noinline__ double solve_general(const cx<float>* z32, const Cand* kk, double te, uint8_t* flag) {
     cx<double> zz[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) zz[i] = mk<double>(z32[i].re, z32[i].im);
     bool w2 = true;
     const EpochOut<double> o2 = solve_epoch<double>(zeta64(*kk, te), kk->d, kk->q, zz, w2, nullptr, kResolveCubic);
-    if (A_row) A_row[e] = o2.A;
-    if (f_row) f_row[e] = (uint8_t)(o2.flag | FLAG_FP64 | why);
-    if (!chi2) return 0.0;
-    const double r = (fe - o2.A) * we;
+    *flag = o2.flag;
+    return o2.A;
+}
+
+// An FP64 re-solve's results: magnification and flags when the row pointers are given (MIXED: the
+// FP64 bit and the triggers beside the solver's own flags); returns the chi^2 term from the FP64
+// flux fe and weight we = 1/sigma.
+template <int MODE>
+__device__ __forceinline__ double store_resolved(double A, uint8_t flag, uint32_t why, double fe, double we,
+                                                 double* A_row, uint8_t* f_row, int e) {
+    if (A_row) A_row[e] = A;
+    if (f_row) f_row[e] = MODE == SBLM_MIXED ? (uint8_t)(flag | FLAG_FP64 | why) : flag;
+    const double r = (fe - A) * we;
     return r * r;
 }
 
-// Where MIXED work goes. Epochs to re-solve in FP64 are appended to `queue` (slots taken with one
-// atomic per warp, so that a later pass re-solves them in full warps; an epoch that finds the queue
-// full is re-solved in place, so the capacity is a speed choice only). Every epoch's chi^2 term is
-// stored in the candidate's row of the dense term array (the FP32 ones here, the FP64 ones by the
-// re-solve, wherever it runs), and the row is summed afterwards in a fixed order: a MIXED chi^2
+// Where MIXED and FP64 work goes. Epochs to re-solve in FP64 are appended to `queue` (slots taken
+// with one atomic per warp, so that a later pass re-solves them side by side; an epoch that finds
+// the queue full is re-solved in place, so the capacity is a speed choice only). Every epoch's chi^2
+// term is stored in the candidate's row of the dense term array (the others here, the re-solved ones
+// by the re-solve, wherever it runs), and the row is summed afterwards in a fixed order: the chi^2
 // does not depend on the order in which the queue filled. `term_row` is the candidate's row
 // (epoch e at term_row[e]); null when no chi^2 is wanted.
 struct DeferSink {
@@ -128,95 +132,137 @@ struct DeferSink {
     unsigned queue_cap;
 };
 
+// One warp's share of the queued epochs [0, n): groups of five lanes take them six at a time, warp
+// `w` of `n_w` starting at epoch 6 w. `cand(c)` is candidate c, `data(c, e)` the epoch's time, flux and
+// 1/sigma, and `store(c, e, A, flag, why, fe, we)` takes the result (one lane per epoch). Every lane
+// of the warp calls it.
+struct EpochData {
+    double t, flux, w;
+};
+template <class CandFn, class DataFn, class StoreFn>
+__device__ __forceinline__ void resolve_queue(const Deferred* __restrict__ queue, unsigned n, unsigned w, unsigned n_w,
+                                              CandFn cand, DataFn data, StoreFn store) {
+    const int lane = threadIdx.x & 31, grp = lane / kResolveLanes, r = lane - grp * kResolveLanes;
+    for (unsigned first = w * kResolvePerWarp; first < n; first += n_w * kResolvePerWarp) {
+        const unsigned i = first + grp;
+        const bool valid = grp < kResolvePerWarp && i < n;
+        const Deferred& q = queue[valid ? i : first];
+        const int c = q.c, e = q.e;
+        const Cand k = cand(c);
+        const EpochData ed = data(c, e);
+        double A;
+        const bool done = resolve_group(q.z[r], valid, zeta64(k, ed.t), k.d, k.q, &A);
+        if (valid && r == 0) {
+            uint8_t flag = 0;
+            if (!done) A = solve_general(q.z, &k, ed.t, &flag);
+            store(c, e, A, flag, q.why, ed.flux, ed.w);
+        }
+        __syncwarp();
+    }
+}
+
 // The thread's epochs [e0, e1) of candidate k (all lanes of a warp run `seg` iterations so that
-// MIXED can reserve queue slots warp-wide). Writes A and flags when the row pointers are given.
-// FP64 and FP32: returns the thread's chi^2 over its epochs, accumulated in FP64 in epoch order.
-// MIXED: writes each epoch's chi^2 term to term_row (CHI2) and returns 0; `c_tag` is the candidate
+// queue slots can be reserved warp-wide). Writes A and flags when the row pointers are given.
+// FP32: returns the thread's chi^2 over its epochs, accumulated in FP64 in epoch order. MIXED and
+// FP64: writes each epoch's chi^2 term to term_row (CHI2) and returns 0; `c_tag` is the candidate
 // index recorded in its queue entries.
+// FP64 solves the quintic in FP32 too: its roots tell images from spurious ones unless a trigger
+// (refine_trigger, wider than MIXED's) sends the epoch to the re-solve, and the images are refined in
+// FP64 (refine_images). 32 epochs of three images cost a warp about 200 FP64 instructions instead of
+// some 6000 of an FP64 root iteration over the union of its lanes' sweeps.
 template <int MODE, bool CHI2, bool STAGED>
 __device__ __forceinline__ double eval_run(const Cand& k, bool valid, int c_tag, int e0, int e1, int seg,
                                            const LCView& lc, double* A_row, uint8_t* f_row, const DeferSink& sink,
                                            double* term_row) {
     double chi = 0.0;
-    if constexpr (MODE == SBLM_FP64) {
-        cx<double> z[5];
-        bool warm = false;
-        for (int e = e0; valid && e < e1; ++e) {
-            const double te = STAGED ? lc.s_t[e] : lc.t[e];
-            const EpochOut<double> o = solve_epoch<double>(zeta64(k, te), k.d, k.q, z, warm);
+    const float t0h = (float)k.t0, t0l = (float)(k.t0 - (double)t0h);
+    const float itE = (float)k.inv_tE, sa = (float)k.sa, ca = (float)k.ca, u0 = (float)k.u0;
+    const float d = (float)k.d, q = (float)k.q;
+    const unsigned lane = threadIdx.x & 31u;
+    const bool refined = MODE == SBLM_FP64 && refine_lens(d, q);
+    cx<float> z[5];
+    bool warm = false;
+    for (int it = 0; it < seg; ++it) {
+        const int e = e0 + it;
+        const bool act = valid && e < e1;
+        bool defer = false;
+        uint8_t why = 0;
+        if constexpr (MODE == SBLM_FP64) {
+            if (act) {
+                const double te = STAGED ? lc.s_t[e] : lc.t[e];
+                const cx<double> zd = zeta64(k, te);
+                const cx<float> zeta = mk<float>((float)zd.re, (float)zd.im);
+                Root<float> rp[5];
+                unsigned images = 0;
+                EpochOut<float> o =
+                    solve_epoch<float>(zeta, d, q, z, warm, nullptr, Tol<float>::cubic, rp, &images);
+                double A = 0.0;
+                defer = refine_trigger(o) || !refined || !refine_source(zeta, d);
+                if (!defer) defer = !refine_images(rp, images, zd, k.d, k.q, &A);
+                if (!defer) {
+                    if (A_row) A_row[e] = A;
+                    if (f_row) f_row[e] = 0;
+                    if (CHI2) {
+                        const double fe = STAGED ? lc.s_f[e] : lc.flux[e];
+                        const double we = STAGED ? lc.s_w[e] : 1.0 / lc.sigma[e];
+                        const double r = (fe - A) * we;
+                        term_row[e] = r * r;
+                    }
+                }
+            }
+        } else if (act) {
+            float4 ep;
+            if (STAGED) {
+                ep = lc.s_ep[e];
+            } else {
+                const double te = lc.t[e];
+                const float th = (float)te;
+                ep = make_float4(th, (float)(te - (double)th), CHI2 ? (float)lc.flux[e] : 0.f,
+                                 CHI2 ? (float)(1.0 / lc.sigma[e]) : 0.f);
+            }
+            const float tau = diff_ff(ep.x, ep.y, t0h, t0l) * itE;
+            const cx<float> zeta = mk<float>(tau * sa + u0 * ca, -tau * ca + u0 * sa);
+            EpochOut<float> o = solve_epoch<float>(zeta, d, q, z, warm);
+            o.flag = mixed_trigger_flags(o);
+            if (MODE == SBLM_MIXED) defer = o.flag != 0;
+            why = o.flag;
             if (A_row) A_row[e] = o.A;
             if (f_row) f_row[e] = o.flag;
-            if (CHI2) {
-                const double fe = STAGED ? lc.s_f[e] : lc.flux[e];
-                const double we = STAGED ? lc.s_w[e] : 1.0 / lc.sigma[e];
-                const double r = (fe - o.A) * we;
-                chi += r * r;
+            if (CHI2 && !defer) {
+                const double r = (double)((ep.z - o.A) * ep.w);
+                if (MODE == SBLM_MIXED)
+                    term_row[e] = r * r;
+                else
+                    chi += r * r;
             }
         }
-    } else {
-        const float t0h = (float)k.t0, t0l = (float)(k.t0 - (double)t0h);
-        const float itE = (float)k.inv_tE, sa = (float)k.sa, ca = (float)k.ca, u0 = (float)k.u0;
-        const float d = (float)k.d, q = (float)k.q;
-        const unsigned lane = threadIdx.x & 31u;
-        cx<float> z[5];
-        bool warm = false;
-        for (int it = 0; it < seg; ++it) {
-            const int e = e0 + it;
-            const bool act = valid && e < e1;
-            bool defer = false;
-            uint8_t why = 0;
-            if (act) {
-                float4 ep;
-                if (STAGED) {
-                    ep = lc.s_ep[e];
-                } else {
-                    const double te = lc.t[e];
-                    const float th = (float)te;
-                    ep = make_float4(th, (float)(te - (double)th), CHI2 ? (float)lc.flux[e] : 0.f,
-                                     CHI2 ? (float)(1.0 / lc.sigma[e]) : 0.f);
-                }
-                const float tau = diff_ff(ep.x, ep.y, t0h, t0l) * itE;
-                const cx<float> zeta = mk<float>(tau * sa + u0 * ca, -tau * ca + u0 * sa);
-                EpochOut<float> o = solve_epoch<float>(zeta, d, q, z, warm);
-                o.flag = mixed_trigger_flags(o);
-                if (MODE == SBLM_MIXED) defer = o.flag != 0;
-                why = o.flag;
-                if (A_row) A_row[e] = o.A;
-                if (f_row) f_row[e] = o.flag;
-                if (CHI2 && !defer) {
-                    const double r = (double)((ep.z - o.A) * ep.w);
-                    if (MODE == SBLM_MIXED)
-                        term_row[e] = r * r;
-                    else
-                        chi += r * r;
-                }
-            }
-            if constexpr (MODE == SBLM_MIXED) {
-                // one atomic per warp reserves queue slots for the lanes that defer
-                const unsigned b = __ballot_sync(0xffffffffu, defer);
-                if (b) {
-                    const int leader = __ffs(b) - 1;
-                    unsigned base = 0;
-                    if ((int)lane == leader) base = atomicAdd(sink.queue_count, (unsigned)__popc(b));
-                    base = __shfl_sync(0xffffffffu, base, leader);
-                    if (defer) {
-                        const unsigned slot = base + (unsigned)__popc(b & ((1u << lane) - 1u));
-                        if (slot < sink.queue_cap) {
-                            Deferred& qd = sink.queue[slot];
+        if constexpr (MODE != SBLM_FP32) {
+            // one atomic per warp reserves queue slots for the lanes that defer
+            const unsigned b = __ballot_sync(0xffffffffu, defer);
+            if (b) {
+                const int leader = __ffs(b) - 1;
+                unsigned base = 0;
+                if ((int)lane == leader) base = atomicAdd(sink.queue_count, (unsigned)__popc(b));
+                base = __shfl_sync(0xffffffffu, base, leader);
+                if (defer) {
+                    const unsigned slot = base + (unsigned)__popc(b & ((1u << lane) - 1u));
+                    if (slot < sink.queue_cap) {
+                        Deferred& qd = sink.queue[slot];
 #pragma unroll
-                            for (int i = 0; i < 5; ++i) qd.z[i] = z[i];
-                            qd.c = c_tag;
-                            qd.e = e;
-                            qd.why = why;
-                        } else {  // queue full: re-solve here, from the FP64 data
-                            const double te = lc.t[e];
-                            const double fe = CHI2 ? lc.flux[e] : 0.0, we = CHI2 ? 1.0 / lc.sigma[e] : 0.0;
-                            cx<float> zc[5];  // a copy, so that z's address is never taken and z stays in registers
+                        for (int i = 0; i < 5; ++i) qd.z[i] = z[i];
+                        qd.c = c_tag;
+                        qd.e = e;
+                        qd.why = why;
+                    } else {  // queue full: re-solve here, from the FP64 data
+                        const double te = lc.t[e];
+                        cx<float> zc[5];  // a copy, so that z's address is never taken and z stays in registers
 #pragma unroll
-                            for (int i = 0; i < 5; ++i) zc[i] = z[i];
-                            const double tm = resolve_fp64(zc, why, &k, te, fe, we, A_row, f_row, e, CHI2);
-                            if (CHI2) term_row[e] = tm;
-                        }
+                        for (int i = 0; i < 5; ++i) zc[i] = z[i];
+                        uint8_t flag;
+                        const double A = solve_general(zc, &k, te, &flag);
+                        const double fe = CHI2 ? lc.flux[e] : 0.0, we = CHI2 ? 1.0 / lc.sigma[e] : 0.0;
+                        const double tm = store_resolved<MODE>(A, flag, why, fe, we, A_row, f_row, e);
+                        if (CHI2) term_row[e] = tm;
                     }
                 }
             }
@@ -225,7 +271,7 @@ __device__ __forceinline__ double eval_run(const Cand& k, bool valid, int c_tag,
     return chi;
 }
 
-// MIXED: sum of a candidate's term row over the lanes of its group of G threads (G a power of two
+// MIXED and FP64: sum of a candidate's term row over the lanes of its group of G threads (G a power of two
 // <= 32, groups aligned within the warp): lane g adds epochs g, g + G, ... in order, then a fixed
 // butterfly combines the lanes; every lane of the group gets the sum. All lanes of the warp call it.
 __device__ __forceinline__ double term_row_sum(const double* __restrict__ row, int n_ep, int g, int G, bool valid) {

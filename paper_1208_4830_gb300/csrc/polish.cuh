@@ -15,7 +15,7 @@
 #pragma once
 
 #include "blend.cuh"
-#include "forward_run.cuh"
+#include "polish_run.cuh"
 
 namespace sblm {
 
