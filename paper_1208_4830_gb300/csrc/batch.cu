@@ -394,8 +394,9 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
                             const double* e = Pc + (size_t)s_idx[0] * n_par;
                             for (int j = 0; j < n_par; ++j) Pn[j] = e[j];
                         }
-                        for (int k = threadIdx.x; k < n_pop / 2; k += blockDim.x)
-                            offspring_pair(c, gen, Pc, s_idx, s_pmut, k, Pn);
+                        // two lanes per pairing, whole warps
+                        for (int i = threadIdx.x; (i & ~31) / 2 < n_pop / 2; i += blockDim.x)
+                            offspring_pair<2>(c, gen, Pc, s_idx, s_pmut, i / 2, i & 1, i / 2 < n_pop / 2, Pn);
                     }
                     __syncthreads();
                 }

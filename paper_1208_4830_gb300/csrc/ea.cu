@@ -2,12 +2,13 @@
 // sblm_ea_generation.
 //
 // One generation after its fitness evaluation takes two launches:
-//   rank_kernel      one block: stable bitonic sort of (chi^2, row) in shared memory, archive of
+//   rank_kernel      one block: stable bitonic sort of (chi^2, row), archive of
 //                    the best ever, stagnation check; on a restart it also writes the sort keys
 //                    of the fresh population;
-//   offspring_kernel one thread per reproductive pairing: tournament selection, weighting
+//   offspring_kernel two or eight lanes per reproductive pairing: tournament selection, weighting
 //                    matrix, Eq. (rep1)/(rep2), creep and jump mutation, elitism in row 0; on a
 //                    restart instead one thread per element of the fresh population.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -88,10 +89,15 @@ __global__ void __launch_bounds__(kRankThreads)
     }
 }
 
-// grid row blockIdx.y is population y of a batch (strides as in rank_kernel)
-__global__ void offspring_kernel(EAConst c, int gen, const double* __restrict__ P, const int* __restrict__ order,
-                                 const EACtrl* __restrict__ ctrl, const uint64_t* __restrict__ keys,
-                                 double* __restrict__ P_next) {
+// grid row blockIdx.y is population y of a batch (strides as in rank_kernel); L lanes per pairing. What
+// bounds it is the FP64 pipe (about 60 instructions per gene of a pairing, 19 cycles each per SM) beside
+// the integer work of the tournaments' draws: 156 us for 32 populations of 4096 with one thread per
+// pairing (2048 warps, 14 per SM), 92 us with two.
+template <int L>
+__global__ void __launch_bounds__(256, 4)
+    offspring_kernel(EAConst c, int gen, const double* __restrict__ P, const int* __restrict__ order,
+                     const EACtrl* __restrict__ ctrl, const uint64_t* __restrict__ keys,
+                     double* __restrict__ P_next) {
     {
         const size_t b = blockIdx.y, m = (size_t)c.n_pop * c.n_par;
         P += b * m;
@@ -104,15 +110,14 @@ __global__ void offspring_kernel(EAConst c, int gen, const double* __restrict__ 
     if (ctrl->restart) {  // uniform over the grid row
         __shared__ uint64_t tile[kInitTile];
         const int m = c.n_pop * c.n_par;
-        block_init_values(c, gen + 1, keys, m, P_next, blockIdx.x * blockDim.x, m, tile, kInitTile);
+        block_init_values(c, gen + 1, keys, m, P_next, blockIdx.x * blockDim.x, gridDim.x * blockDim.x, tile,
+                          kInitTile);
         return;
     }
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k == 0) {  // elitism: the fittest row survives unmutated
-        const double* e = P + (size_t)order[0] * c.n_par;
-        for (int j = 0; j < c.n_par; ++j) P_next[j] = e[j];
-    }
-    if (k < c.n_pop / 2) offspring_pair(c, gen, P, order, ctrl->p_mut_used, k, P_next);  // ceil((N_pop-1)/2)
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, k = i / L, n_pairs = c.n_pop / 2;  // ceil((N_pop-1)/2)
+    if (i < c.n_par) P_next[i] = P[(size_t)order[0] * c.n_par + i];  // elitism: the fittest row survives unmutated
+    if ((i & ~31) / L >= n_pairs) return;  // whole warps
+    offspring_pair<L>(c, gen, P, order, ctrl->p_mut_used, k, i % L, k < n_pairs, P_next);
 }
 
 int blocks_for(int n, int b) { return (n + b - 1) / b; }
@@ -175,8 +180,17 @@ cudaError_t launch_rank(const EAConst& c, int gen, const double* chi2, const dou
 
 cudaError_t launch_offspring(const EAConst& c, int gen, const double* P, const int* order, const EACtrl* ctrl,
                              const uint64_t* keys, double* P_next, cudaStream_t s, int n_pops) {
-    const int m = c.n_pop * c.n_par;
-    offspring_kernel<<<dim3(blocks_for(m, 256), n_pops), 256, 0, s>>>(c, gen, P, order, ctrl, keys, P_next);
+    // enough blocks for one element per thread of a fresh population, and for L lanes per pairing:
+    // eight while the pairings alone do not fill the GPU (a lane then draws an eighth of the tournaments
+    // and mutates one gene), else two (six genes on eight lanes leave a quarter of the FP64 pipe idle)
+    const long pairs = (long)(c.n_pop / 2) * n_pops;
+    const bool wide = pairs * 2 < 32L * 4 * device_sm_count();
+    const int L = wide ? 8 : 2;
+    const dim3 grid(blocks_for(std::max(c.n_pop * c.n_par, (c.n_pop / 2) * L), 256), n_pops);
+    if (wide)
+        offspring_kernel<8><<<grid, 256, 0, s>>>(c, gen, P, order, ctrl, keys, P_next);
+    else
+        offspring_kernel<2><<<grid, 256, 0, s>>>(c, gen, P, order, ctrl, keys, P_next);
     return cudaGetLastError();
 }
 

@@ -47,27 +47,44 @@ __device__ __forceinline__ double init_value(const EAConst& c, uint64_t gen, uin
     return (pos < 2 * n_pairs && (pos & 1)) ? __dsub_rn(1.0, x) : x;
 }
 
-// Appendix A, "Selection": parent rank = min of n_tourn uniform draws from {0..N_pop-1}
-__device__ __forceinline__ int tournament(const EAConst& c, uint64_t gen, uint64_t slot) {
+// Appendix A, "Selection": parent rank = min of n_tourn uniform draws from {0..N_pop-1}, the draws
+// shared by the L lanes of an aligned group (all lanes of the warp call it). The integer draw is
+// monotonic in the word's top 32 bits, so their minimum gives the smallest draw.
+template <int L>
+__device__ __forceinline__ int tournament(const EAConst& c, uint64_t gen, uint64_t slot, int lane) {
     uint32_t best = 0xffffffffu;
-    u64x4 w{};
-    for (int j = 0; j < c.n_tourn; ++j) {
-        if ((j & 3) == 0) w = philox4x64(gen, OP_SELECT, slot, (uint64_t)(j >> 2), c.seed, c.stream);
-        const uint32_t r = uniform_int(w.x[j & 3], (uint32_t)c.n_pop);
-        best = r < best ? r : best;
+    for (int b = lane; 4 * b < c.n_tourn; b += L) {
+        const u64x4 w = philox4x64(gen, OP_SELECT, slot, (uint64_t)b, c.seed, c.stream);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (4 * b + j < c.n_tourn) best = min(best, (uint32_t)(w.x[j] >> 32));
     }
-    return (int)best;
+#pragma unroll
+    for (int o = L / 2; o > 0; o >>= 1) best = min(best, __shfl_xor_sync(0xffffffffu, best, o));
+    return (int)uniform_int((uint64_t)best << 32, (uint32_t)c.n_pop);
 }
 
-// Appendix A, "Creep and jump mutation" of gene j of population row `row`
+// the draw u01(x) < p as an integer comparison: (x >> 11) < ceil(p 2^53)
+__device__ __forceinline__ uint64_t jump_threshold(double p_mut) { return (uint64_t)ceil(p_mut * 0x1.0p53); }
+
+// v clamped to [0, 1] by its bits (NaN and -0 become 0, as fmin(fmax(v, 0), 1) gives)
+__device__ __forceinline__ double clamp_unit(double v) {
+    const long long b = __double_as_longlong(v);
+    if (b < 0 || b > 0x7ff0000000000000ll) return 0.0;
+    return b > 0x3ff0000000000000ll ? 1.0 : v;
+}
+
+// Appendix A, "Creep and jump mutation" of gene j of population row `row`. The FP64 pipe takes a warp
+// instruction per 64 cycles and bounds the offspring kernel with the draws, so both creep directions
+// share their operations, and the clamp and the jump test run on the integer pipe.
 __device__ __forceinline__ double mutate_gene(const EAConst& c, uint64_t gen, uint64_t row, uint64_t j, double p,
-                                              double p_mut) {
+                                              uint64_t p_jump) {
     const u64x4 w = philox4x64(gen, OP_MUT, row, j, c.seed, c.stream);
     const double X = exp(__dmul_rn(kLnEps, u01(w.x[0])));
-    double v = top_bit(w.x[1]) ? __dadd_rn(p, __dmul_rn(__dsub_rn(1.0, p), X)) : __dsub_rn(p, __dmul_rn(p, X));
-    v = fmin(fmax(v, 0.0), 1.0);
-    if (u01(w.x[2]) < p_mut) v = u01(w.x[3]);
-    return v;
+    const bool up = top_bit(w.x[1]);
+    const double step = __dmul_rn(up ? __dsub_rn(1.0, p) : p, X);
+    const double v = __dadd_rn(p, up ? step : -step);
+    return (w.x[2] >> 11) < p_jump ? u01(w.x[3]) : clamp_unit(v);
 }
 
 // Appendix A, "Stagnation checks", applied by one thread after the ranking of generation t.
@@ -102,51 +119,163 @@ __device__ __forceinline__ int stagnation_update(sblm_ea_state& s, const EAConst
     return 0;
 }
 
-// stable ascending order of (key, index) pairs: NaN fitness becomes +inf
-__device__ __forceinline__ bool pair_less(double ka, int ia, double kb, int ib) {
-    return ka < kb || (ka == kb && ia < ib);
-}
-
 // ---------------------------------------------------------------------------------------------
 // Block-level building blocks, shared by the single-population kernels and the persistent
 // batched fitter. Every thread of the calling block must call them (they hold barriers).
 // ---------------------------------------------------------------------------------------------
 
+// fitness as an unsigned integer in the same order (NaN as +inf, -0 as 0), and back
+__device__ __forceinline__ uint64_t order_key(double v) {
+    uint64_t b = (uint64_t)__double_as_longlong(v);
+    if ((b << 1) > 0xffe0000000000000ull) b = 0x7ff0000000000000ull;
+    if ((b << 1) == 0) b = 0;
+    return (b >> 63) ? ~b : b | 0x8000000000000000ull;
+}
+__device__ __forceinline__ double order_value(uint64_t k) {
+    return __longlong_as_double((long long)((k >> 63) ? k & 0x7fffffffffffffffull : ~k));
+}
+__device__ __forceinline__ bool pair_less(uint64_t ka, int ia, uint64_t kb, int ib) {
+    return ka < kb || (ka == kb && ia < ib);
+}
+
+// Ascending bitonic sort of n = E T (key, index) pairs by the block's first T threads (T a power of two,
+// 32 <= T <= blockDim.x), thread t holding elements t E .. t E + E - 1. Strides below E stay in
+// registers, strides below 32 E are warp shuffles, and only the longer ones go through shared memory
+// (bkey, bidx: n each, element e of thread t at e T + t, so consecutive threads touch consecutive
+// words). Every thread of the block calls it. Keys are integers: a comparison of doubles would run on
+// the FP64 pipe. Ranking 32 populations of 4096 (a block each): 175 us with every stage on doubles in
+// shared memory behind a barrier (78 stages), 41 us with 15 such stages on integers.
+template <int E>
+__device__ __forceinline__ void block_sort(uint64_t (&key)[E], int (&idx)[E], int T, uint64_t* bkey, int* bidx) {
+    const int t = threadIdx.x, n = E * T;
+    for (int k = 2; k <= n; k <<= 1) {
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= 32 * E) {
+                const int x = j / E;
+                if (t < T) {
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        bkey[e * T + t] = key[e];
+                        bidx[e * T + t] = idx[e];
+                    }
+                }
+                __syncthreads();
+                if (t < T) {
+                    const bool low = !(t & x);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const uint64_t ok = bkey[e * T + (t ^ x)];
+                        const int oi = bidx[e * T + (t ^ x)];
+                        const bool up = ((t * E + e) & k) == 0;
+                        if (pair_less(ok, oi, key[e], idx[e]) == (up == low)) {
+                            key[e] = ok;
+                            idx[e] = oi;
+                        }
+                    }
+                }
+                __syncthreads();
+            } else if (j >= E) {
+                if (t < T) {  // whole warps
+                    const int x = j / E;
+                    const bool low = !(t & x);
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        const uint64_t ok = __shfl_xor_sync(0xffffffffu, key[e], x);
+                        const int oi = __shfl_xor_sync(0xffffffffu, idx[e], x);
+                        const bool up = ((t * E + e) & k) == 0;
+                        if (pair_less(ok, oi, key[e], idx[e]) == (up == low)) {
+                            key[e] = ok;
+                            idx[e] = oi;
+                        }
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int jj = E / 2; jj > 0; jj >>= 1) {
+                    if (jj != j) continue;
+#pragma unroll
+                    for (int e = 0; e < E; ++e) {
+                        if (e & jj) continue;
+                        const bool up = ((t * E + e) & k) == 0;
+                        if (pair_less(key[e + jj], idx[e + jj], key[e], idx[e]) == up) {
+                            const uint64_t tk = key[e];
+                            key[e] = key[e + jj];
+                            key[e + jj] = tk;
+                            const int ti = idx[e];
+                            idx[e] = idx[e + jj];
+                            idx[e + jj] = ti;
+                        }
+                    }
+                }
+            }
+        }
+    }
+}
+
+template <int E>
+__device__ __forceinline__ void block_rank_regs(const double* chi2, int n_pop, int n2, int T, double* skey, int* sidx) {
+    uint64_t key[E];
+    int idx[E];
+    const int t = threadIdx.x;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = t * E + e;
+        const bool in = t < T && i < n_pop;
+        key[e] = in ? order_key(chi2[i]) : ~0ull;
+        idx[e] = in ? i : 0x7fffffff;
+    }
+    block_sort<E>(key, idx, T, reinterpret_cast<uint64_t*>(skey), sidx);
+    if (t < T) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = t * E + e;
+            if (i < n2) {
+                skey[i] = i < n_pop ? order_value(key[e]) : INFINITY;
+                sidx[i] = idx[e];
+            }
+        }
+    }
+    __syncthreads();
+}
+
 // (fitness, row) pairs of the population in shared memory, NaN as +inf, padded to n2 (a power
-// of two) with (+inf, INT_MAX), then sorted ascending by a bitonic network
+// of two) with (+inf, INT_MAX), sorted ascending (ties by row): skey and sidx hold n2 entries
 __device__ __forceinline__ void block_rank(const double* __restrict__ chi2, int n_pop, int n2, double* skey,
                                            int* sidx) {
+    // threads in use: the largest power of two that gives each at least one element
+    int T = 32;
+    while (2 * T <= (int)blockDim.x && 2 * T <= n2) T <<= 1;
+    switch (max(1, n2 / T)) {
+        case 1: return block_rank_regs<1>(chi2, n_pop, n2, T, skey, sidx);
+        case 2: return block_rank_regs<2>(chi2, n_pop, n2, T, skey, sidx);
+        case 4: return block_rank_regs<4>(chi2, n_pop, n2, T, skey, sidx);
+        case 8: return block_rank_regs<8>(chi2, n_pop, n2, T, skey, sidx);
+    }
+    // more than eight elements per thread (small blocks of the batched fitter): all in shared memory
+    uint64_t* bkey = reinterpret_cast<uint64_t*>(skey);
     for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-        if (i < n_pop) {
-            const double v = chi2[i];
-            skey[i] = isnan(v) ? INFINITY : v;
-            sidx[i] = i;
-        } else {
-            skey[i] = INFINITY;
-            sidx[i] = 0x7fffffff;
-        }
+        bkey[i] = i < n_pop ? order_key(chi2[i]) : ~0ull;
+        sidx[i] = i < n_pop ? i : 0x7fffffff;
     }
     __syncthreads();
     for (int k = 2; k <= n2; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
             for (int i = threadIdx.x; i < n2; i += blockDim.x) {
                 const int l = i ^ j;
-                if (l > i) {
-                    const bool up = (i & k) == 0;
-                    const bool greater = pair_less(skey[l], sidx[l], skey[i], sidx[i]);
-                    if (greater == up) {
-                        const double tk = skey[i];
-                        skey[i] = skey[l];
-                        skey[l] = tk;
-                        const int ti = sidx[i];
-                        sidx[i] = sidx[l];
-                        sidx[l] = ti;
-                    }
+                if (l > i && pair_less(bkey[l], sidx[l], bkey[i], sidx[i]) == ((i & k) == 0)) {
+                    const uint64_t tk = bkey[i];
+                    bkey[i] = bkey[l];
+                    bkey[l] = tk;
+                    const int ti = sidx[i];
+                    sidx[i] = sidx[l];
+                    sidx[l] = ti;
                 }
             }
             __syncthreads();
         }
     }
+    for (int i = threadIdx.x; i < n2; i += blockDim.x) skey[i] = i < n_pop ? order_value(bkey[i]) : INFINITY;
+    __syncthreads();
 }
 
 // One thread's bookkeeping after the ranking of generation `gen`: archive of the best ever,
@@ -165,30 +294,35 @@ __device__ __forceinline__ int block_bookkeeping(const EAConst& c, int gen, doub
 }
 
 // Reproductive pairing k of generation `gen` (Appendix A, "Selection", "Reproduction",
-// "Creep and jump mutation"): two tournament parents from the ranked population (order[r] is
-// the row of rank r), the weighting-matrix mode and diagonal, Eq. (rep1)/(rep2), then creep and
-// jump of both children into rows 1 + 2k and 2 + 2k of P_next (the second dropped past N_pop).
+// "Creep and jump mutation") by the L lanes of an aligned group (lane 0 .. L - 1; all lanes of the
+// warp call it, `valid` false beyond the last pairing): two tournament parents from the ranked
+// population (order[r] is the row of rank r), the weighting-matrix mode and diagonal,
+// Eq. (rep1)/(rep2), then creep and jump of both children into rows 1 + 2k and 2 + 2k of P_next (the
+// second dropped past N_pop). The lanes share the tournaments' draws and the genes.
+template <int L>
 __device__ __forceinline__ void offspring_pair(const EAConst& c, int gen, const double* __restrict__ P,
-                                               const int* __restrict__ order, double p_mut, int k,
-                                               double* __restrict__ P_next) {
+                                               const int* __restrict__ order, double p_mut, int k, int lane,
+                                               bool valid, double* __restrict__ P_next) {
     const int n_par = c.n_par;
     const uint64_t g = (uint64_t)gen;
-    const int ra = tournament(c, g, 2 * (uint64_t)k);
-    const int rb = tournament(c, g, 2 * (uint64_t)k + 1);
+    const int ra = tournament<L>(c, g, 2 * (uint64_t)k, lane);
+    const int rb = tournament<L>(c, g, 2 * (uint64_t)k + 1, lane);
+    if (!valid) return;
     const double* pa = P + (size_t)order[ra] * n_par;
     const double* pb = P + (size_t)order[rb] * n_par;
     const uint32_t mode = uniform_int(philox4x64(g, OP_MODE, (uint64_t)k, 0, c.seed, c.stream).x[0], 3u);
+    const uint64_t p_jump = jump_threshold(p_mut);
     const int row1 = 1 + 2 * k, row2 = 2 + 2 * k;
-    for (int j = 0; j < n_par; ++j) {
+    for (int j = lane; j < n_par; j += L) {
         const uint64_t w = philox4x64(g, OP_F, (uint64_t)k, (uint64_t)j, c.seed, c.stream).x[0];
         const double f = mode == 0 ? u01(w) : (mode == 1 ? (double)top_bit(w) : 1.0);
         const double omf = __dsub_rn(1.0, f);
         const double a = pa[j], b = pb[j];
         const double c1 = __dadd_rn(__dmul_rn(a, f), __dmul_rn(b, omf));
         const double c2 = __dadd_rn(__dmul_rn(b, f), __dmul_rn(a, omf));
-        P_next[(size_t)row1 * n_par + j] = mutate_gene(c, g, (uint64_t)row1, (uint64_t)j, c1, p_mut);
+        P_next[(size_t)row1 * n_par + j] = mutate_gene(c, g, (uint64_t)row1, (uint64_t)j, c1, p_jump);
         if (row2 < c.n_pop)
-            P_next[(size_t)row2 * n_par + j] = mutate_gene(c, g, (uint64_t)row2, (uint64_t)j, c2, p_mut);
+            P_next[(size_t)row2 * n_par + j] = mutate_gene(c, g, (uint64_t)row2, (uint64_t)j, c2, p_jump);
     }
 }
 
