@@ -14,6 +14,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <vector>
 
 #include "../../include/sblm_cnn.h"
@@ -188,7 +189,7 @@ __device__ void block_sort256(T* s) {
 // input normalisation of one curve, thread j = bin j: asinh(10 (F / median - 1)) / 3 and the mask
 // (T = float for training curves, double for observed ones)
 template <typename T>
-__device__ void normalise_block(T F, bool kept, int n_kept, float* xrow, T* s_v) {
+__device__ float2 normalise_block(T F, bool kept, int n_kept, T* s_v) {
     const int j = threadIdx.x;
     s_v[j] = kept ? F : T(INFINITY);
     __syncthreads();
@@ -198,15 +199,29 @@ __device__ void normalise_block(T F, bool kept, int n_kept, float* xrow, T* s_v)
     if (!(med > T(0) && isfinite(med))) med = T(1);
     float2 o = make_float2(0.f, 0.f);
     if (kept) o = make_float2((float)(asinh(T(10) * (F / med - T(1))) / T(3)), 1.f);
-    reinterpret_cast<float2*>(xrow)[j] = o;
+    return o;
+}
+
+// The network input in BF16 as the first convolution's products read it: [B][260][2], two zero positions on
+// either side of a sample. Position j of sample i, by thread j of 256.
+constexpr int kInputRow = kBins + 4;
+__device__ __forceinline__ void store_input(__nv_bfloat16* xb, int i, int j, float2 v) {
+    uint32_t* row = reinterpret_cast<uint32_t*>(xb) + (size_t)i * kInputRow;
+    row[j + 2] = pack_bf2(v.x, v.y);
+    if (j < 4) row[j < 2 ? j : kBins + j] = 0u;
 }
 
 // ------------------------------------------------------------------------------------------
 // kernels around the network
 // ------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(kBins) input_kernel(const float* x, __nv_bfloat16* xb) {
+    store_input(xb, blockIdx.x, threadIdx.x, reinterpret_cast<const float2*>(x)[(size_t)blockIdx.x * kBins + threadIdx.x]);
+}
+// ctr[0], ctr[1]: the network's step and the first step of the run; ctr[2]: the generator's step
 __global__ void set_counter_kernel(int64_t* ctr, int64_t step, int64_t first) {
     ctr[0] = step;
     ctr[1] = first;
+    ctr[2] = step;
 }
 __global__ void advance_kernel(int64_t* ctr) { ctr[0] += 1; }
 
@@ -231,7 +246,7 @@ __global__ void init_kernel(float* w, uint64_t seed) {
     w[idx] = v;
 }
 
-// training sample i of step ctr[0]: parameters (window units), noise settings, targets
+// training sample i of step *ctr: parameters (window units), noise settings, targets
 __global__ void gen_kernel(uint64_t seed, const int64_t* ctr, int B, double forced_frac, double* theta, double* aux,
                            float* y) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -303,7 +318,7 @@ __global__ void gen_kernel(uint64_t seed, const int64_t* ctr, int B, double forc
 // normalisation run in FP32 (the FP64 pipe is slow and the inputs are FP32); the mask decisions
 // compare the 53-bit uniforms in FP64.
 __global__ void __launch_bounds__(kBins) prep_kernel(const double* A, const double* aux, uint64_t seed,
-                                                      const int64_t* ctr, float* x) {
+                                                      const int64_t* ctr, float* x, __nv_bfloat16* xb) {
     __shared__ float s_v[kBins];
     const int i = blockIdx.x, j = threadIdx.x;
     const uint64_t step = (uint64_t)ctr[0];
@@ -322,7 +337,9 @@ __global__ void __launch_bounds__(kBins) prep_kernel(const double* A, const doub
         n = kBins;
     }
     const float F = (float)A[(size_t)i * kBins + j] * (1.f + (float)ax[0] * z);
-    normalise_block<float>(F, kept, n, x + (size_t)i * 2 * kBins, s_v);
+    const float2 v = normalise_block<float>(F, kept, n, s_v);
+    if (x) reinterpret_cast<float2*>(x)[(size_t)i * kBins + j] = v;
+    if (xb) store_input(xb, i, j, v);
 }
 
 // observed curve blockIdx.x resampled to the bins over its own span (thread = bin)
@@ -380,7 +397,7 @@ __global__ void __launch_bounds__(kBins) bin_kernel(const double* t, const doubl
     const bool kept = sw > 0.0;
     const double F = kept ? swf / sw : 0.0;
     const int n_kept = __syncthreads_count(kept);
-    normalise_block<double>(F, kept, n_kept, x + (size_t)lc * 2 * kBins, s_v);
+    reinterpret_cast<float2*>(x)[(size_t)lc * kBins + j] = normalise_block<double>(F, kept, n_kept, s_v);
     if (j == 0) {
         window[2 * lc] = 0.5 * (tmin + tmax);
         window[2 * lc + 1] = 0.5 * span;
@@ -451,21 +468,49 @@ struct AdamArgs {
     float* v;
     double lr0, b1, b2, eps, wd;
     int n_steps, warmup;
-    int64_t t;           // 1-based step when ctr is null
-    const int64_t* ctr;  // else t = ctr[0] + 1
+    int64_t t;              // 1-based step
+    const double* scalars;  // the step's learning rate and bias corrections, or null: computed from t
 };
+
+// the learning rate of 1-based step t and the bias corrections 1 / (1 - beta^t): a cosine and two powers, some
+// 400 instructions of the FP64 pipe
+__device__ __forceinline__ double adam_scalar(const AdamArgs& ad, int64_t t, int k) {
+    if (k == 0) return lr_at(t, ad.n_steps, ad.warmup, ad.lr0);
+    return 1.0 / (1.0 - pow(k == 1 ? ad.b1 : ad.b2, (double)t));
+}
+// the scalars of step ctr[0] + 1, once instead of in every block of the update
+__global__ void adam_scalars_kernel(AdamArgs ad, const int64_t* ctr, double* out) {
+    if (threadIdx.x < 3) out[threadIdx.x] = adam_scalar(ad, ctr[0] + 1, threadIdx.x);
+}
+
+// 1/x and sqrt(x) of positive doubles to a few 2^-53: a hardware approximation and Newton steps (the
+// library's division and square root are some 70 instructions of the FP64 pipe, which bounded this
+// kernel with the bias corrections' powers in every block: 49 us for 326,156 parameters, 32 us with both
+// taken out); sqrt(0) = 0
+__device__ __forceinline__ double reciprocal(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+__device__ __forceinline__ double square_root(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    // y <- y + y e / 2 + 3 y e^2 / 8, e = 1 - x y^2, then one correction of s = x y
+    const double e = fma(-x * y, y, 1.0);
+    y = fma(y * e, fma(0.375, e, 0.5), y);
+    const double s = x * y;
+    const double t = fma(0.5 * y, fma(-s, s, x), s);
+    return x > 0.0 && isfinite(t) ? t : sqrt(x);
+}
 
 // gradient = sum of the partials in split order (or grad_in); optional AdamW step and BF16 copies
 __global__ void update_kernel(PartTab tab, const float* grad_in, float* grad_out, AdamArgs ad, float* w,
                               __nv_bfloat16* wb, __nv_bfloat16* wbt) {
     // the step's learning rate and bias corrections 1 / (1 - beta^t), once per block
     __shared__ double s_sc[3];
-    if (ad.on && threadIdx.x == 0) {
-        const int64_t t = ad.ctr ? ad.ctr[0] + 1 : ad.t;
-        s_sc[0] = lr_at(t, ad.n_steps, ad.warmup, ad.lr0);
-        s_sc[1] = 1.0 / (1.0 - pow(ad.b1, (double)t));
-        s_sc[2] = 1.0 / (1.0 - pow(ad.b2, (double)t));
-    }
+    if (ad.on && threadIdx.x < 3)
+        s_sc[threadIdx.x] = ad.scalars ? ad.scalars[threadIdx.x] : adam_scalar(ad, ad.t, threadIdx.x);
     __syncthreads();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= kNParams) return;
@@ -480,6 +525,7 @@ __global__ void update_kernel(PartTab tab, const float* grad_in, float* grad_out
         const float* p = tab.p[l] + r;
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
         int s = 0;
+#pragma unroll 4
         for (; s + 4 <= z; s += 4) {
             a0 += p[(size_t)s * cnt];
             a1 += p[(size_t)(s + 1) * cnt];
@@ -498,7 +544,7 @@ __global__ void update_kernel(PartTab tab, const float* grad_in, float* grad_out
         const double v = ad.b2 * (double)ad.v[idx] + (1.0 - ad.b2) * (double)g * g;
         const double mh = m * s_sc[1];
         const double vh = v * s_sc[2];
-        wd = wd - lr * mh / (sqrt(vh) + ad.eps);
+        wd = wd - lr * mh * reciprocal(square_root(vh) + ad.eps);
         ad.m[idx] = (float)m;
         ad.v[idx] = (float)v;
         wv = (float)wd;
@@ -524,48 +570,51 @@ __global__ void propose_kernel(const float* out, const double* window, int n_lc,
 // ------------------------------------------------------------------------------------------
 // tensor-core epilogues
 // ------------------------------------------------------------------------------------------
+__device__ __forceinline__ float4 add4(float4 v, const float* b) {
+    return make_float4(v.x + b[0], v.y + b[1], v.z + b[2], v.w + b[3]);
+}
+__device__ __forceinline__ void store_bf4(__nv_bfloat16* p, float a, float b, float c, float d) {
+    *reinterpret_cast<uint2*>(p) = make_uint2(pack_bf2(a, b), pack_bf2(c, d));
+}
 struct EpiAct {  // z = acc + bias; keep z (training) and GELU(z) in BF16
     const float* bias;
     float* z;
     __nv_bfloat16* h;
     int M, N;
-    __device__ void operator()(int m, int n, float v0, float v1, int) const {
+    __device__ void operator()(int m, int n, float4 v, int) const {
         if (m >= M || n >= N) return;
-        v0 += bias[n];
-        v1 += bias[n + 1];
+        v = add4(v, bias + n);
         const size_t i = (size_t)m * N + n;
-        if (z) *reinterpret_cast<float2*>(z + i) = make_float2(v0, v1);
-        *reinterpret_cast<uint32_t*>(h + i) = pack_bf2(gelu(v0), gelu(v1));
+        if (z) *reinterpret_cast<float4*>(z + i) = v;
+        store_bf4(h + i, gelu(v.x), gelu(v.y), gelu(v.z), gelu(v.w));
     }
 };
 struct EpiOut {  // network output: acc + bias, FP32
     const float* bias;
     float* out;
     int M, N;
-    __device__ void operator()(int m, int n, float v0, float v1, int) const {
+    __device__ void operator()(int m, int n, float4 v, int) const {
         if (m >= M || n >= N) return;
-        *reinterpret_cast<float2*>(out + (size_t)m * N + n) = make_float2(v0 + bias[n], v1 + bias[n + 1]);
+        *reinterpret_cast<float4*>(out + (size_t)m * N + n) = add4(v, bias + n);
     }
 };
-struct EpiDgrad {  // gradient of the pre-activation: acc * GELU'(z), BF16
+struct EpiDgrad {  // gradient of the pre-activation: acc * GELU'(z), BF16; row m at m * ld + off
     const float* z;
     __nv_bfloat16* dz;
-    int M, N;
-    __device__ void operator()(int m, int n, float v0, float v1, int) const {
+    int M, N, ld, off;
+    __device__ void operator()(int m, int n, float4 v, int) const {
         if (m >= M || n >= N) return;
-        const size_t i = (size_t)m * N + n;
-        const float2 zz = *reinterpret_cast<const float2*>(z + i);
-        *reinterpret_cast<uint32_t*>(dz + i) = pack_bf2(v0 * gelu_grad(zz.x), v1 * gelu_grad(zz.y));
+        const size_t i = (size_t)m * ld + off + n;
+        const float4 zz = *reinterpret_cast<const float4*>(z + i);
+        store_bf4(dz + i, v.x * gelu_grad(zz.x), v.y * gelu_grad(zz.y), v.z * gelu_grad(zz.z), v.w * gelu_grad(zz.w));
     }
 };
 struct EpiPart {  // weight-gradient partial of split z
     float* part;
     int M, N;
-    __device__ void operator()(int m, int n, float v0, float v1, int z) const {
+    __device__ void operator()(int m, int n, float4 v, int z) const {
         if (m >= M || n >= N) return;
-        float* p = part + ((size_t)z * M + m) * N + n;
-        p[0] = v0;
-        if (n + 1 < N) p[1] = v1;
+        *reinterpret_cast<float4*>(part + ((size_t)z * M + m) * N + n) = v;  // every N is a multiple of 4
     }
 };
 
@@ -573,37 +622,44 @@ struct EpiPart {  // weight-gradient partial of split z
 // host side
 // ------------------------------------------------------------------------------------------
 struct Split {
-    int z = 1, tps = 1;
+    int z = 1, ksplit = 0;  // splits of the reduction, and its length in each
 };
 
+constexpr int kSplitUnit = 32;
+
 Split split_for(int M, int N, int K, int sms) {
-    const int nt = (K + BK - 1) / BK;
+    const int nt = (K + kSplitUnit - 1) / kSplitUnit;
     const int tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
     int want = std::max(1, (sms + tiles - 1) / tiles);
     want = std::min(want, nt);
+    const int tps = (nt + want - 1) / want;
     Split s;
-    s.tps = (nt + want - 1) / want;
-    s.z = (nt + s.tps - 1) / s.tps;
+    s.z = (nt + tps - 1) / tps;
+    s.ksplit = tps * kSplitUnit;
     return s;
 }
 
-template <bool AK, bool BKM, class LA, class LB, class EP>
-cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int N, int K, Split sp, cudaStream_t s) {
-    auto kern = gemm_kernel<AK, BKM, LA, LB, EP>;
-    // opt in to the two-stage tile ring (> 48 KB) once per device and instantiation; the first
+template <bool AK, bool BKM, int STAGES, class LA, class LB, class EP>
+cudaError_t launch_gemm(const LA& la, const LB& lb, const EP& ep, int M, int N, int K, Split sp, cudaStream_t s) {
+    auto kern = gemm_kernel<AK, BKM, STAGES, LA, LB, EP>;
+    // opt in to the tile ring (> 48 KB) once per device and instantiation; the first
     // launch of a sequence runs outside any stream capture
-    cudaError_t e = raise_smem_limit((const void*)kern, kGemmSmem);
+    cudaError_t e = raise_smem_limit((const void*)kern, gemm_smem(STAGES));
     if (e != cudaSuccess) return e;
     dim3 grid((M + BM - 1) / BM, (N + BN - 1) / BN, sp.z);
-    kern<<<grid, kGemmThreads, kGemmSmem, s>>>(la, lb, ep, M, N, K, sp.tps);
+    kern<<<grid, kGemmThreads, gemm_smem(STAGES), s>>>(la, lb, ep, M, N, K, sp.ksplit);
     return cudaGetLastError();
 }
 template <bool AK, bool BKM, class LA, class LB, class EP>
+cudaError_t gemm(const LA& la, const LB& lb, const EP& ep, int M, int N, int K, Split sp, cudaStream_t s) {
+    return launch_gemm<AK, BKM, kDeep>(la, lb, ep, M, N, K, sp, s);
+}
+template <bool AK, bool BKM, int STAGES = kShallow, class LA, class LB, class EP>
 cudaError_t gemm1(const LA& la, const LB& lb, const EP& ep, int M, int N, int K, cudaStream_t s) {
     Split sp;
     sp.z = 1;
-    sp.tps = (K + BK - 1) / BK;
-    return gemm<AK, BKM>(la, lb, ep, M, N, K, sp, s);
+    sp.ksplit = K;
+    return launch_gemm<AK, BKM, STAGES>(la, lb, ep, M, N, K, sp, s);
 }
 
 // lay out consecutive 256-byte aligned pieces of one region; with base == nullptr only sizes
@@ -624,7 +680,7 @@ int sm_count() { return device_sm_count(); }
 struct Net {
     int B = 0;
     bool train = false;
-    const float* x = nullptr;
+    __nv_bfloat16* xb = nullptr;  // [B][260][2], carved unless the caller brings its own
     __nv_bfloat16 *wb = nullptr, *wbt = nullptr;
     __nv_bfloat16 *h1, *h2, *h3, *h4, *h5;
     float *z1 = nullptr, *z2 = nullptr, *z3 = nullptr, *z4 = nullptr, *z5 = nullptr;
@@ -644,12 +700,13 @@ void wgrad_shape(int l, int B, int* M, int* N, int* K) {
     *K = l < 4 ? B * Lo[l] : B;
 }
 
-Net carve_net(Carver& c, int B, bool train, int sms) {
+Net carve_net(Carver& c, int B, bool train, int sms, bool own_input = true) {
     Net n;
     n.B = B;
     n.train = train;
     n.wb = c.take<__nv_bfloat16>(kNParams);
     n.wbt = c.take<__nv_bfloat16>(kNParams);
+    n.xb = own_input ? c.take<__nv_bfloat16>((size_t)B * kInputRow * 2) : nullptr;
     n.h1 = c.take<__nv_bfloat16>((size_t)B * 256 * 64);
     n.h2 = c.take<__nv_bfloat16>((size_t)B * 128 * 64);
     n.h3 = c.take<__nv_bfloat16>((size_t)B * 64 * 64);
@@ -679,6 +736,25 @@ Net carve_net(Carver& c, int B, bool train, int sms) {
     return n;
 }
 
+// The stream that draws training batches beside the network, and its fork and join events: one set per
+// device, kept until the process exits; used under the call lock
+struct SideStream {
+    cudaStream_t stream = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr;
+};
+
+sblm_status side_stream(SideStream** out) {
+    static std::map<int, SideStream>* sets = new std::map<int, SideStream>();
+    int dev = 0;
+    SBLM_CUDA(cudaGetDevice(&dev));
+    SideStream& s = (*sets)[dev];
+    if (!s.stream) SBLM_CUDA(cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking));
+    if (!s.fork) SBLM_CUDA(cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming));
+    if (!s.join) SBLM_CUDA(cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming));
+    *out = &s;
+    return SBLM_OK;
+}
+
 #define CNN_TRY(call)                              \
     do {                                           \
         cudaError_t e_ = (call);                   \
@@ -689,19 +765,30 @@ Net carve_net(Carver& c, int B, bool train, int sms) {
 cudaError_t net_forward(const Net& n, const float* w, cudaStream_t s) {
     const int B = n.B;
     const __nv_bfloat16* wbt = n.wbt;
-    CNN_TRY((gemm1<true, true>(InputIm2col{n.x, B}, DenseBF{wbt + kOffH[0], 64, 10, 10, -1},
+    CNN_TRY((gemm1<true, true>(InputCols{n.xb, B}, DenseBFAny{wbt + kOffH[0], 64, 10, 10},
                                EpiAct{w + kOffH[0] + 640, n.z1, n.h1, B * 256, 64}, B * 256, 64, 10, s)));
-    CNN_TRY((gemm1<true, true>(Im2col{n.h1, B, 256, 128, 2}, DenseBF{wbt + kOffH[1], 64, 320, 320, -1},
+    CNN_TRY((gemm1<true, true>(Im2col{n.h1, B, 7}, DenseBF{wbt + kOffH[1], 64, 320, 320, false},
                                EpiAct{w + kOffH[1] + 20480, n.z2, n.h2, B * 128, 64}, B * 128, 64, 320, s)));
-    CNN_TRY((gemm1<true, true>(Im2col{n.h2, B, 128, 64, 2}, DenseBF{wbt + kOffH[2], 64, 320, 320, -1},
+    CNN_TRY((gemm1<true, true>(Im2col{n.h2, B, 6}, DenseBF{wbt + kOffH[2], 64, 320, 320, false},
                                EpiAct{w + kOffH[2] + 20480, n.z3, n.h3, B * 64, 64}, B * 64, 64, 320, s)));
-    CNN_TRY((gemm1<true, true>(Im2col{n.h3, B, 64, 32, 2}, DenseBF{wbt + kOffH[3], 64, 320, 320, -1},
+    CNN_TRY((gemm1<true, true>(Im2col{n.h3, B, 5}, DenseBF{wbt + kOffH[3], 64, 320, 320, false},
                                EpiAct{w + kOffH[3] + 20480, n.z4, n.h4, B * 32, 64}, B * 32, 64, 320, s)));
-    CNN_TRY((gemm1<true, true>(DenseBF{n.h4, B, 2048, 2048, -1}, DenseBF{wbt + kOffH[4], 128, 2048, 2048, -1},
+    CNN_TRY((gemm1<true, true, kDeep>(DenseBF{n.h4, B, 2048, 2048, false}, DenseBF{wbt + kOffH[4], 128, 2048, 2048, false},
                                EpiAct{w + kOffH[4] + 262144, n.z5, n.h5, B, 128}, B, 128, 2048, s)));
-    CNN_TRY((gemm1<true, true>(DenseBF{n.h5, B, 128, 128, -1}, DenseBF{wbt + kOffH[5], 12, 128, 128, -1},
+    CNN_TRY((gemm1<true, true>(DenseBF{n.h5, B, 128, 128, false}, DenseBF{wbt + kOffH[5], 12, 128, 128, false},
                                EpiOut{w + kOffH[5] + 1536, n.out, B, 12}, B, 12, 128, s)));
     return cudaSuccess;
+}
+
+// gradient of the pre-activations z of a stride-2 convolution's input [B][2 Lo][64] from that of its
+// output: one product per parity of the input position
+cudaError_t conv_input_gradient(const __nv_bfloat16* dz_out, int B, int log_lo, const __nv_bfloat16* w, const float* z,
+                                __nv_bfloat16* dz, cudaStream_t s) {
+    const int M = B << log_lo;
+    CNN_TRY((gemm1<true, true>(ConvGrad<0>{dz_out, B, log_lo}, ConvWT<0>{w}, EpiDgrad{z, dz, M, 64, 128, 0}, M, 64, 192,
+                               s)));
+    return gemm1<true, true>(ConvGrad<1>{dz_out, B, log_lo}, ConvWT<1>{w}, EpiDgrad{z, dz, M, 64, 128, 64}, M, 64, 128,
+                             s);
 }
 
 // backward pass from n.dout: weight-gradient partials of every layer
@@ -709,32 +796,29 @@ cudaError_t net_backward(const Net& n, cudaStream_t s) {
     const int B = n.B;
     const __nv_bfloat16* wb = n.wb;
     // dense 128 -> 12
-    CNN_TRY((gemm<false, false>(DenseBF{n.h5, B, 128, 128, 128}, DenseF32{n.dout, B, 12, 12},
+    CNN_TRY((gemm<false, false>(DenseBF{n.h5, B, 128, 128, true}, DenseF32{n.dout, B, 12, 12},
                                 EpiPart{n.part[5], 129, 12}, 129, 12, B, n.sp[5], s)));
-    CNN_TRY((gemm1<true, true>(DenseF32{n.dout, B, 12, 12}, DenseBF{wb + kOffH[5], 128, 12, 12, -1},
-                               EpiDgrad{n.z5, n.dz5, B, 128}, B, 128, 12, s)));
+    CNN_TRY((gemm1<true, true>(DenseF32{n.dout, B, 12, 12}, DenseBFAny{wb + kOffH[5], 128, 12, 12},
+                               EpiDgrad{n.z5, n.dz5, B, 128, 128, 0}, B, 128, 12, s)));
     // dense 2048 -> 128
-    CNN_TRY((gemm<false, false>(DenseBF{n.h4, B, 2048, 2048, 2048}, DenseBF{n.dz5, B, 128, 128, -1},
+    CNN_TRY((gemm<false, false>(DenseBF{n.h4, B, 2048, 2048, true}, DenseBF{n.dz5, B, 128, 128, false},
                                 EpiPart{n.part[4], 2049, 128}, 2049, 128, B, n.sp[4], s)));
-    CNN_TRY((gemm1<true, true>(DenseBF{n.dz5, B, 128, 128, -1}, DenseBF{wb + kOffH[4], 2048, 128, 128, -1},
-                               EpiDgrad{n.z4, n.dz4, B, 2048}, B, 2048, 128, s)));
+    CNN_TRY((gemm1<true, true>(DenseBF{n.dz5, B, 128, 128, false}, DenseBF{wb + kOffH[4], 2048, 128, 128, false},
+                               EpiDgrad{n.z4, n.dz4, B, 2048, 2048, 0}, B, 2048, 128, s)));
     // conv 4 (64 -> 32 positions)
-    CNN_TRY((gemm<false, false>(Im2colT{n.h3, B, 64, 32, 2}, DenseBF{n.dz4, B * 32, 64, 64, -1},
+    CNN_TRY((gemm<false, false>(Im2colT{n.h3, B, 5}, DenseBF{n.dz4, B * 32, 64, 64, false},
                                 EpiPart{n.part[3], 321, 64}, 321, 64, B * 32, n.sp[3], s)));
-    CNN_TRY((gemm1<true, true>(Col2im{n.dz4, B, 64, 32, 2}, ConvWT{wb + kOffH[3]}, EpiDgrad{n.z3, n.dz3, B * 64, 64},
-                               B * 64, 64, 320, s)));
+    CNN_TRY(conv_input_gradient(n.dz4, B, 5, wb + kOffH[3], n.z3, n.dz3, s));
     // conv 3 (128 -> 64)
-    CNN_TRY((gemm<false, false>(Im2colT{n.h2, B, 128, 64, 2}, DenseBF{n.dz3, B * 64, 64, 64, -1},
+    CNN_TRY((gemm<false, false>(Im2colT{n.h2, B, 6}, DenseBF{n.dz3, B * 64, 64, 64, false},
                                 EpiPart{n.part[2], 321, 64}, 321, 64, B * 64, n.sp[2], s)));
-    CNN_TRY((gemm1<true, true>(Col2im{n.dz3, B, 128, 64, 2}, ConvWT{wb + kOffH[2]},
-                               EpiDgrad{n.z2, n.dz2, B * 128, 64}, B * 128, 64, 320, s)));
+    CNN_TRY(conv_input_gradient(n.dz3, B, 6, wb + kOffH[2], n.z2, n.dz2, s));
     // conv 2 (256 -> 128)
-    CNN_TRY((gemm<false, false>(Im2colT{n.h1, B, 256, 128, 2}, DenseBF{n.dz2, B * 128, 64, 64, -1},
+    CNN_TRY((gemm<false, false>(Im2colT{n.h1, B, 7}, DenseBF{n.dz2, B * 128, 64, 64, false},
                                 EpiPart{n.part[1], 321, 64}, 321, 64, B * 128, n.sp[1], s)));
-    CNN_TRY((gemm1<true, true>(Col2im{n.dz2, B, 256, 128, 2}, ConvWT{wb + kOffH[1]},
-                               EpiDgrad{n.z1, n.dz1, B * 256, 64}, B * 256, 64, 320, s)));
+    CNN_TRY(conv_input_gradient(n.dz2, B, 7, wb + kOffH[1], n.z1, n.dz1, s));
     // conv 1 (input)
-    CNN_TRY((gemm<false, false>(InputIm2colT{n.x, B}, DenseBF{n.dz1, B * 256, 64, 64, -1},
+    CNN_TRY((gemm<false, false>(InputCols{n.xb, B}, DenseBF{n.dz1, B * 256, 64, 64, false},
                                 EpiPart{n.part[0], 11, 64}, 11, 64, B * 256, n.sp[0], s)));
     return cudaSuccess;
 }
@@ -753,6 +837,11 @@ constexpr int kUpdBlocks = (kNParams + kUpdThreads - 1) / kUpdThreads;
 
 cudaError_t launch_cast(const float* w, __nv_bfloat16* wb, __nv_bfloat16* wbt, cudaStream_t s) {
     cast_kernel<<<kUpdBlocks, kUpdThreads, 0, s>>>(w, wb, wbt);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_input(const float* x, const Net& n, cudaStream_t s) {
+    input_kernel<<<n.B, kBins, 0, s>>>(x, n.xb);
     return cudaGetLastError();
 }
 
@@ -775,15 +864,15 @@ Gen carve_gen(Carver& c, int B, int precision, bool own_theta) {
     g.y = c.take<float>((size_t)B * 6);
     g.grid = c.take<double>(kBins);
     g.mixed = c.take<unsigned char>(mixed_scratch_bytes(precision, B, kBins, false));
-    g.ctr = c.take<int64_t>(2);
+    g.ctr = c.take<int64_t>(4);
     return g;
 }
 
-// draw a batch at step ctr[0]: parameters, forward model, noise and normalisation
-cudaError_t launch_gen(const Gen& g, int B, int precision, double forced_frac, uint64_t seed, float* x, float* y,
-                       cudaStream_t s) {
+// draw a batch at step ctr[2]: parameters, forward model, noise and normalisation
+cudaError_t launch_gen(const Gen& g, int B, int precision, double forced_frac, uint64_t seed, float* x, __nv_bfloat16* xb,
+                       float* y, cudaStream_t s) {
     // one warp per block: the caustic-aimed samples (an FP64 root iteration each) spread over the SMs
-    gen_kernel<<<(B + 31) / 32, 32, 0, s>>>(seed, g.ctr, B, forced_frac, g.theta, g.aux, y);
+    gen_kernel<<<(B + 31) / 32, 32, 0, s>>>(seed, g.ctr + 2, B, forced_frac, g.theta, g.aux, y);
     CNN_TRY(cudaGetLastError());
     ForwardArgs fa{};
     fa.src = g.theta;
@@ -795,7 +884,7 @@ cudaError_t launch_gen(const Gen& g, int B, int precision, double forced_frac, u
     fa.G = choose_group(B, kBins);
     fa.mixed = g.mixed;
     CNN_TRY(launch_forward(fa, s));
-    prep_kernel<<<B, kBins, 0, s>>>(g.A, g.aux, seed, g.ctr, x);
+    prep_kernel<<<B, kBins, 0, s>>>(g.A, g.aux, seed, g.ctr + 2, x, xb);
     return cudaGetLastError();
 }
 
@@ -811,7 +900,7 @@ sblm_status check_train_params(const sblm_cnn_train_params* p) {
     return SBLM_OK;
 }
 
-AdamArgs adam_args(const sblm_cnn_train_params* p, float* state, int64_t t, const int64_t* ctr) {
+AdamArgs adam_args(const sblm_cnn_train_params* p, float* state, int64_t t, const double* scalars) {
     AdamArgs a{};
     a.on = true;
     a.m = state;
@@ -824,7 +913,7 @@ AdamArgs adam_args(const sblm_cnn_train_params* p, float* state, int64_t t, cons
     a.n_steps = p->n_steps;
     a.warmup = p->warmup;
     a.t = t;
-    a.ctr = ctr;
+    a.scalars = scalars;
     return a;
 }
 
@@ -841,7 +930,6 @@ InferScratch carve_infer(Carver& c, int n, int n_seed, Net* net) {
     sc.window = c.take<double>((size_t)n * 2);
     sc.genes = c.take<double>((size_t)n * std::max(1, n_seed) * 6);
     Net nn = carve_net(c, n, false, 1);
-    nn.x = sc.x;
     sc.wb = nn.wb;
     sc.wbt = nn.wbt;
     sc.act = nn.h1;
@@ -871,6 +959,7 @@ cudaError_t launch_seed_rows(const double* t, const double* flux, const double* 
     bin_kernel<<<n_lc, kBins, 0, s>>>(t, flux, sigma, offsets, sc.x, sc.window);
     CNN_TRY(cudaGetLastError());
     CNN_TRY(launch_cast(weights, net.wb, net.wbt, s));
+    CNN_TRY(launch_input(sc.x, net, s));
     CNN_TRY(net_forward(net, weights, s));
     const long long total = (long long)n_lc * n_seed;
     if (total > 0) {
@@ -981,7 +1070,7 @@ sblm_status sblm_cnn_make_batch(uint64_t seed, int64_t step, int32_t batch, doub
     set_counter_kernel<<<1, 1, 0, s>>>(g.ctr, step, step);
     grid_kernel<<<1, kBins, 0, s>>>(g.grid);
     SBLM_CUDA(launch_gen(g, batch, precision, forced_frac, seed, static_cast<float*>(st.dev(i_x)),
-                         static_cast<float*>(st.dev(i_y)), s));
+                         nullptr, static_cast<float*>(st.dev(i_y)), s));
     return st.end();
 }
 
@@ -1039,9 +1128,9 @@ sblm_status sblm_cnn_forward(const float* weights, const float* x, int32_t batch
     SBLM_TRY(st.begin());
     Carver c{static_cast<char*>(st.scratch_ptr(k))};
     Net n = carve_net(c, batch, false, 1);
-    n.x = static_cast<const float*>(st.dev(i_x));
     const float* w = static_cast<const float*>(st.dev(i_w));
     SBLM_CUDA(launch_cast(w, n.wb, n.wbt, s));
+    SBLM_CUDA(launch_input(static_cast<const float*>(st.dev(i_x)), n, s));
     SBLM_CUDA(net_forward(n, w, s));
     SBLM_CUDA(cudaMemcpyAsync(st.dev(i_o), n.out, sizeof(float) * (size_t)batch * 12, cudaMemcpyDeviceToDevice, s));
     SBLM_TRY(check_timeout(s));
@@ -1068,9 +1157,9 @@ sblm_status sblm_cnn_loss_grad(const float* weights, const float* x, const float
     SBLM_TRY(st.begin());
     Carver c{static_cast<char*>(st.scratch_ptr(k))};
     Net n = carve_net(c, batch, true, sms);
-    n.x = static_cast<const float*>(st.dev(i_x));
     float* w = static_cast<float*>(st.dev(i_w));
     SBLM_CUDA(launch_cast(w, n.wb, n.wbt, s));
+    SBLM_CUDA(launch_input(static_cast<const float*>(st.dev(i_x)), n, s));
     SBLM_CUDA(net_forward(n, w, s));
     SBLM_CUDA(launch_loss(n.out, static_cast<const float*>(st.dev(i_y)), batch, n.dout, n.loss_part,
                           static_cast<double*>(st.dev(i_l)), nullptr, nullptr, s));
@@ -1117,30 +1206,52 @@ sblm_status sblm_cnn_train(float* weights, float* adam_state, const sblm_cnn_tra
     SBLM_TRY(st.arg(adam_state, sizeof(float) * 2 * kNParams, true, true, &i_a));
     SBLM_TRY(st.arg(loss_history, loss_history ? sizeof(float) * (size_t)n_run : 0, false, true, &i_h));
     const int B = p->batch, sms = sm_count();
+    const size_t nx = (size_t)B * kInputRow * 2, ny = (size_t)B * 6;
     Carver probe{nullptr};
-    carve_net(probe, B, true, sms);
+    carve_net(probe, B, true, sms, false);
     carve_gen(probe, B, p->precision, true);
-    probe.take<float>((size_t)B * 2 * kBins);
+    probe.take<__nv_bfloat16>(2 * nx);
+    probe.take<float>(2 * ny);
+    probe.take<double>(3);
     const int k = st.scratch(probe.off);
     SBLM_TRY(st.begin());
     Carver c{static_cast<char*>(st.scratch_ptr(k))};
-    Net n = carve_net(c, B, true, sms);
+    Net n = carve_net(c, B, true, sms, false);
     Gen g = carve_gen(c, B, p->precision, true);
-    float* x = c.take<float>((size_t)B * 2 * kBins);
-    n.x = x;
+    __nv_bfloat16* x = c.take<__nv_bfloat16>(2 * nx);  // two batches: the one in training and the next one
+    float* y = c.take<float>(2 * ny);
+    double* scalars = c.take<double>(3);
     float* w = static_cast<float*>(st.dev(i_w));
     float* state = static_cast<float*>(st.dev(i_a));
     float* hist = static_cast<float*>(st.dev(i_h));
+    SideStream* side = nullptr;
+    SBLM_TRY(side_stream(&side));
     set_counter_kernel<<<1, 1, 0, s>>>(g.ctr, first_step, first_step);
     grid_kernel<<<1, kBins, 0, s>>>(g.grid);
     SBLM_CUDA(launch_cast(w, n.wb, n.wbt, s));
-    const AdamArgs ad = adam_args(p, state, 0, g.ctr);
+    const AdamArgs ad = adam_args(p, state, 0, scalars);
     const PartTab tab = part_tab(n);
-    auto enqueue = [&](cudaStream_t q) -> cudaError_t {
-        CNN_TRY(launch_gen(g, B, p->precision, p->forced_frac, p->seed, x, g.y, q));
-        CNN_TRY(net_forward(n, w, q));
-        CNN_TRY(launch_loss(n.out, g.y, B, n.dout, n.loss_part, nullptr, hist, g.ctr, q));
-        CNN_TRY(net_backward(n, q));
+    auto generate = [&](cudaStream_t q, int buf) -> cudaError_t {
+        CNN_TRY(launch_gen(g, B, p->precision, p->forced_frac, p->seed, nullptr, x + buf * nx, y + buf * ny, q));
+        advance_kernel<<<1, 1, 0, q>>>(g.ctr + 2);
+        return cudaGetLastError();
+    };
+    // One step on batch `buf`. The next batch does not depend on the weights: with `more` it is drawn into the
+    // other buffer beside the network's products (the generator keeps the FP32 and FP64 pipes busy, the
+    // products wait on memory): a step of batch 1024 takes 0.55 ms, 0.64 ms one after the other.
+    auto step = [&](cudaStream_t q, int buf, bool more) -> cudaError_t {
+        CNN_TRY(cudaEventRecord(side->fork, q));
+        CNN_TRY(cudaStreamWaitEvent(side->stream, side->fork, 0));
+        adam_scalars_kernel<<<1, 32, 0, side->stream>>>(ad, g.ctr, scalars);
+        CNN_TRY(cudaGetLastError());
+        if (more) CNN_TRY(generate(side->stream, buf ^ 1));
+        CNN_TRY(cudaEventRecord(side->join, side->stream));
+        Net nb = n;
+        nb.xb = x + buf * nx;
+        CNN_TRY(net_forward(nb, w, q));
+        CNN_TRY(launch_loss(nb.out, y + buf * ny, B, nb.dout, nb.loss_part, nullptr, hist, g.ctr, q));
+        CNN_TRY(net_backward(nb, q));
+        CNN_TRY(cudaStreamWaitEvent(q, side->join, 0));
         update_kernel<<<kUpdBlocks, kUpdThreads, 0, q>>>(tab, nullptr, nullptr, ad, w, n.wb, n.wbt);
         CNN_TRY(cudaGetLastError());
         advance_kernel<<<1, 1, 0, q>>>(g.ctr);
@@ -1167,7 +1278,16 @@ sblm_status sblm_cnn_train(float* weights, float* adam_state, const sblm_cnn_tra
     int dev = 0;
     SBLM_CUDA(cudaGetDevice(&dev));
     put(key, dev);
-    for (int i = 0; i < n_run; ++i) SBLM_TRY(run_cached_graph(key, enqueue, s));
+    // two steps (both buffers) per graph while a later step needs the second one's batch, the rest directly
+    auto pair = [&](cudaStream_t q) -> cudaError_t {
+        CNN_TRY(step(q, 0, true));
+        return step(q, 1, true);
+    };
+    SBLM_CUDA(generate(s, 0));
+    int left = n_run;
+    for (; left >= 3; left -= 2) SBLM_TRY(run_cached_graph(key, pair, s));
+    if (left == 2) SBLM_CUDA(step(s, 0, true));
+    SBLM_CUDA(step(s, left == 2 ? 1 : 0, false));
     SBLM_TRY(check_timeout(s));
     return st.end();
 }

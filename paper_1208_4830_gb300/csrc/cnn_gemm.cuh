@@ -3,28 +3,34 @@
 // One tile kernel computes C[M, N] = sum_k A(m, k) B(k, n) with BF16 operands and FP32
 // accumulators held in tensor memory: tcgen05.mma (kind::f16, M = 128, N = 64, K = 16 per
 // instruction) issued by one thread, operands read by the tensor core from shared memory through
-// matrix descriptors, results brought back with tcgen05.ld for the epilogue. Operands are
-// produced by loader functors that return 8 consecutive BF16 values along the operand's
-// contiguous dimension, so the convolution's im2col and its adjoint col2im are never
-// materialised: the loader gathers the rows straight from the activations. Shared memory holds
-// every tile in a no-swizzle core-matrix layout (8 rows x 16 bytes per core matrix): K-major
-// operands (forward and input-gradient products) as 8-row groups of BK/8 core matrices along K;
-// MN-major operands (weight-gradient products, reductions over batch x position, split over K
-// with one FP32 partial per split so the reduction order is fixed) as 8-k groups of core
-// matrices along M or N, read with the instruction descriptor's MN-major bit. In both layouts a
-// core matrix's 16-byte rows are consecutive, so vector v of a tile lands at byte 16 v and each
-// warp stores 512 contiguous bytes (the fetch assigns vectors to threads accordingly). The
-// descriptors' leading-dimension offset is the step between core matrices along K, the
-// stride-dimension offset the step between them along M or N. Two stages: the global loads of the next K-tile overlap the MMAs of the
-// current one, each stage released by an mbarrier that tcgen05.commit arrives on. Every wait is
-// bounded; a wait that gives up sets g_tc_timeout, which the host reads after the call. The
-// give-up decision is made block-wide (__syncthreads_and) before any barrier or .sync.aligned
-// instruction that depends on it: after it no further MMA is issued, the epilogue is skipped, and
-// the block waits for the MMAs already issued (one more commit on a drain barrier) before it
-// frees its tensor memory.
-// The accumulators leave tensor memory through a shared-memory staging tile, so that each warp's
-// epilogue covers one whole 64-column row (coalesced). Two tiles are fetched ahead in registers.
-// Epilogue functors receive two adjacent columns (m, n), (m, n + 1) per call.
+// matrix descriptors, results brought back with tcgen05.ld for the epilogue. Loader functors map
+// (row, column) of an operand to 8 consecutive BF16 values along its contiguous dimension, so the
+// convolution's im2col and its adjoint are never materialised: the loader gathers the rows
+// straight from the activations. K-major operands serve the forward and input-gradient products,
+// MN-major operands (the instruction descriptor's MN-major bit) the weight-gradient products,
+// reductions over batch x position split over K with one FP32 partial per split so the reduction
+// order is fixed.
+//
+// Tiles are rows of 128 bytes (64 values along the contiguous dimension: K-major a row of M or N with 64
+// k, MN-major a k with 64 of M or N) in the 128-byte swizzle: 16-byte chunk c of row r at chunk
+// c ^ (r & 7). Eight lanes copy one row, so a warp touches four whole 128-byte lines: 40 bytes a clock and
+// SM, against 16 for the 16-byte core-matrix columns of the no-swizzle layout, whose gather took one
+// lane a clock and bounded every product (770 cycles per 12 KB, with tcgen05.mma at 160 cycles). The
+// products of a training step of batch 1024 took 0.61 ms so (K-steps of 32 behind block-wide barriers,
+// two tiles ahead through registers, integer divisions in the loaders), 0.32 ms now.
+//
+// The warps have roles, so that no K-step holds a block-wide barrier: warps 0-7 fill a ring of K-tiles
+// (cp.async, zero fill outside the operand, arriving on the stage's `full` barrier when it lands), one
+// thread of warp 8 waits for a full stage, makes it visible to the tensor core and issues its
+// MMAs, and tcgen05.commit arrives on the stage's `empty` barrier. Warps 0-7 then run the epilogue.
+// Positions per sample are powers of two, so rows split by shifts.
+// Every wait is bounded; a wait that gives up sets g_tc_timeout, which the host reads after the call.
+// After a give-up the thread leaves its loop (the waits that depend on it run out as well), the block
+// takes one decision (__syncthreads_and) before the epilogue, skips it, and waits for the MMAs already
+// issued (one more commit on a drain barrier) before it frees its tensor memory.
+// The accumulators leave tensor memory through a shared-memory staging tile, so that half a warp's
+// epilogue covers one whole 64-column row (coalesced). Epilogue functors receive four adjacent columns
+// (m, n .. n + 3) per call.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -36,15 +42,19 @@
 namespace sblm {
 namespace cnn {
 
-constexpr int BM = 128, BN = 64, BK = 32;
-constexpr int kGemmThreads = 256;  // 8 warps: warp w reads accumulator rows 32 (w % 4) .. + 31,
-                                   // columns 32 (w / 4) .. + 31
-constexpr int kStages = 2;
+constexpr int BM = 128, BN = 64, BK = 64;
+constexpr int kProducers = 256;    // warps 0-7 fill the ring and run the epilogue: warp w reads
+                                   // accumulator rows 32 (w % 4) .. + 31, columns 32 (w / 4) .. + 31
+constexpr int kGemmThreads = 288;  // warp 8 issues the MMAs
+// K-tiles in the ring: three leave room for three blocks per SM, which overlap one another's
+// epilogues; eight keep enough copies in flight where a product has one block per SM and many K-steps
+// (weight gradients, the wide dense layer)
+constexpr int kShallow = 3, kDeep = 8;
 constexpr uint32_t kTileA = BM * BK * 2, kTileB = BN * BK * 2;
-constexpr int kEpiLd = BN + 1;  // padded row of the accumulator staging tile (floats)
-constexpr size_t kRing = kStages * (kTileA + kTileB);
-constexpr size_t kEpiBytes = (size_t)BM * kEpiLd * 4;
-constexpr size_t kGemmSmem = (kRing > kEpiBytes ? kRing : kEpiBytes) + 1024;  // + room to align to 1 KB
+constexpr int kEpiLd = BN + 4;  // padded row of the accumulator staging tile (floats)
+// dynamic shared memory: the ring (the epilogue's staging tile reuses it) and room to align it to 1 KB
+constexpr size_t gemm_smem(int stages) { return (size_t)stages * (kTileA + kTileB) + 1024; }
+static_assert(gemm_smem(kShallow) - 1024 >= sizeof(float) * BM * kEpiLd, "the staging tile fits the ring");
 constexpr uint32_t kTmemCols = 64;                                 // FP32 accumulator columns (= BN)
 constexpr int kWaitLimit = 1 << 24;
 
@@ -63,12 +73,12 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// shared-memory matrix descriptor: start address, leading-dimension byte offset (between core
-// matrices along K), stride-dimension byte offset (between 8-row groups), descriptor version 1,
-// no swizzle
+// shared-memory matrix descriptor, 128-byte swizzle: start address, leading-dimension byte offset
+// (MN-major: between blocks of 64 along M or N; not used K-major), stride-dimension byte offset (between
+// groups of 8 rows), descriptor version 1, swizzle mode 2
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
     return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
+           ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
 // instruction descriptor of kind::f16: FP32 accumulator (bits 4-5), BF16 A and B (bits 7-9,
@@ -92,60 +102,94 @@ __device__ __forceinline__ bool mbar_wait(uint32_t addr, uint32_t parity, int li
     return false;
 }
 
-// global -> registers for one tile of ROWS (M or N) x BK. Vector v (8 BF16) is the 16-byte row
-// of core matrix v / 8 at position v % 8: K-major, row group v / BK, k chunk (v % BK) / 8, row
-// v % 8 of the group; MN-major, k group v / ROWS, m (or n) chunk (v % ROWS) / 8, k row v % 8.
+// 16 bytes global -> shared, asynchronous; a null source fills with zeros
+__device__ __forceinline__ void copy16(uint32_t dst, const void* src, const void* any) {
+    const int n = src ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src ? src : any), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ void copy4(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+struct InputCols;
+
+// One tile of ROWS (M or N) x BK into the stage's tile at s, `kc` (a multiple of 16) of its BK along K in
+// use. K-major: row r of ROWS at 128 r. MN-major: for each block of 64 along M or N, row k at 128 k.
+// Loaders of aligned BF16 data give addresses (asynchronous copies), the others values.
 template <bool KMAJ, int ROWS, class L>
-__device__ __forceinline__ void tile_fetch(const L& ld, int mn0, int k0, uint4* reg) {
-    constexpr int per = ROWS * BK / 8 / kGemmThreads;
+__device__ __forceinline__ void tile_load(const L& ld, int mn0, int k0, int kc, unsigned char* s) {
+    if constexpr (std::is_same<L, InputCols>::value) {
+        // rows of ten values, five 4-byte copies each; the rest of the tile was written once (input_tile_init)
+        constexpr int rows = KMAJ ? ROWS : BK;
+        for (int v = threadIdx.x; v < 5 * rows; v += kProducers) {
+            const int r = v / 5, e = v - 5 * r;
+            const void* src = ld.src((KMAJ ? mn0 : k0) + r, e);
+            if (src && (KMAJ || r < kc))
+                copy4(smem_u32(s) + 128u * (uint32_t)r + 16u * (uint32_t)((e >> 2) ^ (r & 7)) + 4u * (uint32_t)(e & 3), src);
+        }
+        return;
+    }
+    constexpr int per = ROWS * BK / 8 / kProducers;
 #pragma unroll
     for (int i = 0; i < per; ++i) {
-        const int v = threadIdx.x + i * kGemmThreads;
-        if (KMAJ) {
-            const int r = (v / BK) * 8 + (v & 7), c = ((v % BK) >> 3) * 8;
-            reg[i] = ld(mn0 + r, k0 + c);
+        const int v = threadIdx.x + i * kProducers, r = v >> 3, c = v & 7;
+        const uint32_t at = 128u * (uint32_t)r + 16u * (uint32_t)(c ^ (r & 7));
+        const int row = KMAJ ? mn0 + r : k0 + r % BK;
+        const int col = KMAJ ? k0 + 8 * c : mn0 + 64 * (r / BK) + 8 * c;
+        if (KMAJ ? 8 * c >= kc : r % BK >= kc) continue;
+        if constexpr (std::is_same<L, InputCols>::value) {
+        } else if constexpr (L::kAsync) {
+            copy16(smem_u32(s) + at, ld.src(row, col), ld.base());
         } else {
-            const int kr = (v / ROWS) * 8 + (v & 7), c = ((v % ROWS) >> 3) * 8;
-            reg[i] = ld(k0 + kr, mn0 + c);
+            *reinterpret_cast<uint4*>(s + at) = ld(row, col);
         }
     }
 }
 
-// registers -> the stage's tile: vector v at byte 16 v
-template <int ROWS>
-__device__ __forceinline__ void tile_store(unsigned char* s, const uint4* reg) {
-    constexpr int per = ROWS * BK / 8 / kGemmThreads;
-#pragma unroll
-    for (int i = 0; i < per; ++i) reinterpret_cast<uint4*>(s)[threadIdx.x + i * kGemmThreads] = reg[i];
-}
-
-// matrix descriptor of the 16-k slice ks of a tile: K-major, core matrices along K 128 bytes
-// apart and 8-row groups (BK/8) * 128 apart; MN-major, 8-k groups (ROWS/8) * 128 apart and
-// core matrices along M or N 128 bytes apart
-template <bool KMAJ, int ROWS>
+// matrix descriptor of the 16-k slice ks of a tile: K-major, 32 bytes along the swizzled rows; MN-major, 16
+// rows down
+template <bool KMAJ>
 __device__ __forceinline__ uint64_t tile_desc(uint32_t base, int ks) {
-    if (KMAJ) return smem_desc(base + (uint32_t)ks * 256, 128, (BK / 8) * 128);
-    return smem_desc(base + (uint32_t)ks * 2 * (ROWS / 8) * 128, (ROWS / 8) * 128, 128);
+    if (KMAJ) return smem_desc(base + (uint32_t)ks * 32, 16, 1024);
+    return smem_desc(base + (uint32_t)ks * 2048, BK * 128, 1024);
 }
 
-// C[M, N] (+ epilogue) over the K-tiles [z * tps, (z + 1) * tps) of split z = blockIdx.z
-template <bool AK, bool BKM, class LA, class LB, class EP>
-__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(LA la, LB lb, EP ep, int M, int N, int K, int tps) {
+__device__ __forceinline__ void mbar_init(uint64_t* b, int count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count));
+}
+__device__ __forceinline__ void commit_mmas(uint64_t* b) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(b)));
+}
+
+// C[M, N] (+ epilogue) over k in [z * ksplit, (z + 1) * ksplit) of split z = blockIdx.z (ksplit a multiple of
+// 32 when there are several)
+template <bool AK, bool BKM, int kStages, class LA, class LB, class EP>
+__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(LA la, LB lb, EP ep, int M, int N, int K, int ksplit) {
     extern __shared__ unsigned char dsmem[];
-    __shared__ __align__(8) uint64_t mbar[kStages];
-    __shared__ __align__(8) uint64_t mbar_drain;  // completes once every MMA issued so far has (give-up path)
+    __shared__ __align__(8) uint64_t full[kStages], empty[kStages];
+    __shared__ __align__(8) uint64_t mbar_drain;  // completes once every MMA issued has
     __shared__ uint32_t s_tmem;
+    constexpr uint32_t kStage = kTileA + kTileB;
     unsigned char* base = reinterpret_cast<unsigned char*>(((uintptr_t)dsmem + 1023) & ~(uintptr_t)1023);
-    unsigned char* sA[kStages] = {base, base + kTileA + kTileB};
-    unsigned char* sB[kStages] = {base + kTileA, base + 2 * kTileA + kTileB};
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
-    const int nt = (K + BK - 1) / BK;
-    const int t_begin = blockIdx.z * tps, t_end = min(nt, t_begin + tps);
+    const int k_begin = blockIdx.z * ksplit, k_end = min(K, k_begin + ksplit);
 
+    if constexpr (std::is_same<LA, InputCols>::value) {
+        // the tile outside the copied values: zeros, and in the weight gradient the bias row's ones (column 10)
+        for (int v = tid; v < kStages * (int)(kTileA / 16); v += kGemmThreads) {
+            const int st = v / (kTileA / 16), i = v % (kTileA / 16), r = i >> 3, c = (i & 7) ^ (r & 7);
+            reinterpret_cast<uint4*>(base + st * kStage)[i] =
+                make_uint4(0u, !AK && r < BK && c == 1 ? 0x3f80u : 0u, 0u, 0u);
+        }
+    }
     if (tid == 0) {
-        for (int s = 0; s < kStages; ++s) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar[s])));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&mbar_drain)));
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(&full[s], kProducers);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&mbar_drain, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) {
@@ -158,77 +202,66 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(LA la, LB lb, EP ep,
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = s_tmem;
 
-    constexpr int kPa = BM * BK / 8 / kGemmThreads, kPb = BN * BK / 8 / kGemmThreads;
-    uint4 ra[2][kPa], rb[2][kPb];
-    uint32_t parity[kStages] = {0u, 0u};
-    bool pending[kStages] = {false, false};
     bool ok = true;
-    // two tiles in flight in registers: tile t + 2 is fetched while the MMAs of tile t run
-    if (t_begin < t_end) {
-        tile_fetch<AK, BM>(la, m0, t_begin * BK, ra[0]);
-        tile_fetch<BKM, BN>(lb, n0, t_begin * BK, rb[0]);
-    }
-    if (t_begin + 1 < t_end) {
-        tile_fetch<AK, BM>(la, m0, (t_begin + 1) * BK, ra[1]);
-        tile_fetch<BKM, BN>(lb, n0, (t_begin + 1) * BK, rb[1]);
-    }
-    // one K-tile through stage ST (a compile-time index, so the register tiles stay in registers)
-    auto step = [&](auto stage, int t) {
-        constexpr int st = decltype(stage)::value;
-        if (pending[st]) {  // the MMAs that read this stage two tiles ago must be done
-            ok = mbar_wait(smem_u32(&mbar[st]), parity[st]) && ok;
-            parity[st] ^= 1u;
-            pending[st] = false;
+    if (tid < kProducers) {
+        int st = 0;
+        uint32_t par = 1;  // the first pass over the ring finds every stage empty
+        for (int k = k_begin; k < k_end; k += BK) {
+            if (k - k_begin >= kStages * BK && !mbar_wait(smem_u32(&empty[st]), par)) {
+                ok = false;
+                break;
+            }
+            unsigned char* s = base + st * kStage;
+            const int kc = min(BK, (k_end - k + 15) & ~15);
+            tile_load<AK, BM>(la, m0, k, kc, s);
+            tile_load<BKM, BN>(lb, n0, k, kc, s + kTileA);
+            if constexpr (LA::kAsync && LB::kAsync) {
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[st])) : "memory");
+            } else {  // plain stores among them: landed and fenced before the arrival
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full[st])) : "memory");
+            }
+            if (++st == kStages) {
+                st = 0;
+                par ^= 1u;
+            }
         }
-        tile_store<BM>(sA[st], ra[st]);
-        tile_store<BN>(sB[st], rb[st]);
-        asm volatile("fence.proxy.async.shared::cta;");
-        asm volatile("tcgen05.fence::before_thread_sync;");
-        ok = __syncthreads_and(ok) != 0;  // one decision for the block: no MMA is issued after a give-up
-        asm volatile("tcgen05.fence::after_thread_sync;");
-        if (tid == 0 && ok) {
-            const uint32_t a0 = smem_u32(sA[st]), b0 = smem_u32(sB[st]);
-#pragma unroll
-            for (int ks = 0; ks < BK / 16; ++ks) {
-                const uint64_t ad = tile_desc<AK, BM>(a0, ks);
-                const uint64_t bd = tile_desc<BKM, BN>(b0, ks);
-                const uint32_t acc = (t > t_begin || ks > 0) ? 1u : 0u;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (tid == kProducers) {
+        int st = 0;
+        uint32_t par = 0;
+        for (int k = k_begin; k < k_end; k += BK) {
+            if (!mbar_wait(smem_u32(&full[st]), par)) {
+                ok = false;
+                break;
+            }
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const uint32_t a0 = smem_u32(base + st * kStage), b0 = a0 + kTileA;
+            const int n_ks = (min(BK, k_end - k) + 15) / 16;
+            for (int ks = 0; ks < n_ks; ++ks) {
+                const uint64_t ad = tile_desc<AK>(a0, ks);
+                const uint64_t bd = tile_desc<BKM>(b0, ks);
+                const uint32_t acc = (k > k_begin || ks > 0) ? 1u : 0u;
                 asm volatile(
                     "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                     " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
                     "l"(ad), "l"(bd), "r"(idesc_f16(!AK, !BKM)), "r"(acc));
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(&mbar[st])));
+            commit_mmas(&empty[st]);
+            if (++st == kStages) {
+                st = 0;
+                par ^= 1u;
+            }
         }
-        pending[st] = ok;
-        if (t + 2 < t_end) {
-            tile_fetch<AK, BM>(la, m0, (t + 2) * BK, ra[st]);
-            tile_fetch<BKM, BN>(lb, n0, (t + 2) * BK, rb[st]);
-        }
-    };
-    for (int t = t_begin; t < t_end; t += 2) {
-        step(std::integral_constant<int, 0>{}, t);
-        if (t + 1 < t_end) step(std::integral_constant<int, 1>{}, t + 1);
+        commit_mmas(&mbar_drain);  // tracks every MMA issued, also after a give-up
+        ok = mbar_wait(smem_u32(&mbar_drain), 0u) && ok;
     }
-    for (int s = 0; s < kStages; ++s)
-        if (pending[s]) {
-            ok = mbar_wait(smem_u32(&mbar[s]), parity[s]) && ok;
-            parity[s] ^= 1u;
-        }
     asm volatile("tcgen05.fence::before_thread_sync;");
     ok = __syncthreads_and(ok) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (!ok) {
-        // a wait gave up: the MMAs issued so far may still be running. Track them all with one more
-        // commit and wait for it (bounded again) before the tensor memory is freed
-        if (tid == 0)
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(&mbar_drain)));
-        mbar_wait(smem_u32(&mbar_drain), 0u);
-        asm volatile("tcgen05.fence::after_thread_sync;");
-    }
-    if (ok && t_end > t_begin) {
+    if (ok && k_end > k_begin && tid < kProducers) {
         float* sE = reinterpret_cast<float*>(base);  // the tile ring is free: every MMA has completed
         const int q = warp & 3, half = warp >> 2;
 #pragma unroll
@@ -244,17 +277,16 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(LA la, LB lb, EP ep,
                   "=r"(r[15])
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;");
-            float* row = sE + (q * 32 + lane) * kEpiLd + col;
+            uint4* row = reinterpret_cast<uint4*>(sE + (q * 32 + lane) * kEpiLd + col);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) row[j] = __uint_as_float(r[j]);
+            for (int j = 0; j < 4; ++j) row[j] = make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
         }
-        __syncthreads();
-        // a warp covers one row's 32 column pairs
+        asm volatile("bar.sync 1, %0;" ::"n"(kProducers) : "memory");  // the epilogue's warps
+        // half a warp covers one row's 16 column quads
 #pragma unroll 4
-        for (int p = tid; p < BM * (BN / 2); p += kGemmThreads) {
-            const int rr = p / (BN / 2), pc = p % (BN / 2);
-            const float* e = sE + rr * kEpiLd + 2 * pc;
-            ep(m0 + rr, n0 + 2 * pc, e[0], e[1], blockIdx.z);
+        for (int p = tid; p < BM * (BN / 4); p += kProducers) {
+            const int rr = p / (BN / 4), pc = p % (BN / 4);
+            ep(m0 + rr, n0 + 4 * pc, *reinterpret_cast<const float4*>(sE + rr * kEpiLd + 4 * pc), blockIdx.z);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -263,22 +295,38 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(LA la, LB lb, EP ep,
 }
 
 // ------------------------------------------------------------------------------------------
-// loaders: operator()(row, col) returns the 8 values at stored (row, col .. col + 7), zero
-// outside the operand
+// loaders: the 8 values at stored (row, col .. col + 7), zero outside the operand: their address
+// (src; kAsync) or the values (operator())
 // ------------------------------------------------------------------------------------------
 
-// dense BF16 matrix [rows][ld]; column `ones_col` (if >= cols) reads as 1 on valid rows
+// a one and seven zeros: the vector that holds the bias row's ones in a weight-gradient operand
+__device__ uint4 g_ones8 = {0x3f80u, 0u, 0u, 0u};
+
+// dense BF16 matrix [rows][ld] whose rows start on 16-byte boundaries (ld and cols multiples of 8); with
+// `ones`, column `cols` reads as 1 on valid rows
 struct DenseBF {
+    static constexpr bool kAsync = true;
     const __nv_bfloat16* p;
-    int rows, cols, ld, ones_col;
+    int rows, cols, ld;
+    bool ones;
+    __device__ const void* base() const { return p; }
+    __device__ const void* src(int r, int c) const {
+        if (r >= rows || c > cols || (c == cols && !ones)) return nullptr;
+        return c == cols ? static_cast<const void*>(&g_ones8) : p + (size_t)r * ld + c;
+    }
+};
+
+// dense BF16 matrix [rows][ld] of any alignment
+struct DenseBFAny {
+    static constexpr bool kAsync = false;
+    const __nv_bfloat16* p;
+    int rows, cols, ld;
     __device__ uint4 operator()(int r, int c) const {
-        if (r >= rows) return make_uint4(0, 0, 0, 0);
-        if (c + 8 <= cols && (ld & 7) == 0) return *reinterpret_cast<const uint4*>(p + (size_t)r * ld + c);
         float v[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
             const int e = c + i;
-            v[i] = e < cols ? __bfloat162float(p[(size_t)r * ld + e]) : (e == ones_col ? 1.f : 0.f);
+            v[i] = (r < rows && e < cols) ? __bfloat162float(p[(size_t)r * ld + e]) : 0.f;
         }
         return pack8(v);
     }
@@ -286,6 +334,7 @@ struct DenseBF {
 
 // dense FP32 matrix [rows][ld], rounded to BF16 on load
 struct DenseF32 {
+    static constexpr bool kAsync = false;
     const float* p;
     int rows, cols, ld;
     __device__ uint4 operator()(int r, int c) const {
@@ -299,98 +348,78 @@ struct DenseF32 {
     }
 };
 
-// im2col of a [B][L][64] BF16 activation for a kernel-5, pad-2 convolution of stride s:
-// row m = b * Lo + l, column k = kk * 64 + c -> h[b][l * s + kk - 2][c]   (K-major A)
+// im2col of a [B][2 Lo][64] BF16 activation for a kernel-5, pad-2 convolution of stride 2, Lo = 2^log_lo:
+// row m = b * Lo + l, column k = kk * 64 + c -> h[b][2 l + kk - 2][c]   (K-major A)
 struct Im2col {
+    static constexpr bool kAsync = true;
     const __nv_bfloat16* h;
-    int B, L, Lo, s;
-    __device__ uint4 operator()(int m, int k) const {
-        if (m >= B * Lo || k >= 5 * 64) return make_uint4(0, 0, 0, 0);
-        const int b = m / Lo, l = m - b * Lo, kk = k >> 6, c = k & 63;
-        const int i = l * s + kk - 2;
-        if (i < 0 || i >= L) return make_uint4(0, 0, 0, 0);
-        return *reinterpret_cast<const uint4*>(h + ((size_t)b * L + i) * 64 + c);
+    int B, log_lo;
+    __device__ const void* base() const { return h; }
+    __device__ const void* src(int m, int k) const {
+        const int b = m >> log_lo, l = m & ((1 << log_lo) - 1);
+        const int i = 2 * l + (k >> 6) - 2;
+        if (b >= B || k >= 5 * 64 || i < 0 || i >= (2 << log_lo)) return nullptr;
+        return h + (((size_t)b << (log_lo + 1)) + i) * 64 + (k & 63);
     }
 };
 
 // the same gather stored MN-major for the weight gradient: row = b * Lo + l, column m = kk * 64 + c,
 // and column 320 reads as 1 (the bias row of the gradient)
 struct Im2colT {
+    static constexpr bool kAsync = true;
     const __nv_bfloat16* h;
-    int B, L, Lo, s;
-    __device__ uint4 operator()(int r, int m) const {
-        if (r >= B * Lo || m > 5 * 64) return make_uint4(0, 0, 0, 0);
-        if (m == 5 * 64) return make_uint4(pack_bf2(1.f, 0.f), 0, 0, 0);
-        const int b = r / Lo, l = r - b * Lo, kk = m >> 6, c = m & 63;
-        const int i = l * s + kk - 2;
-        if (i < 0 || i >= L) return make_uint4(0, 0, 0, 0);
-        return *reinterpret_cast<const uint4*>(h + ((size_t)b * L + i) * 64 + c);
+    int B, log_lo;
+    __device__ const void* base() const { return h; }
+    __device__ const void* src(int r, int m) const {
+        const int b = r >> log_lo, l = r & ((1 << log_lo) - 1);
+        if (b >= B || m > 5 * 64) return nullptr;
+        if (m == 5 * 64) return &g_ones8;
+        const int i = 2 * l + (m >> 6) - 2;
+        if (i < 0 || i >= (2 << log_lo)) return nullptr;
+        return h + (((size_t)b << (log_lo + 1)) + i) * 64 + (m & 63);
     }
 };
 
-// im2col of the FP32 network input [B][256][2] for the first (stride-1) convolution:
-// row m = b * 256 + l, column k = kk * 2 + c < 10   (K-major A)
-struct InputIm2col {
-    const float* x;
+// im2col of the network input for the first (stride-1) convolution, from its BF16 copy with two zero
+// positions on either side of a sample, xb [B][260][2]: row b * 256 + l holds the ten values from position
+// l on, column kk * 2 + c. K-major A of the forward product; MN-major A of the weight gradient, where
+// column 10 reads as 1 (the bias row). src: the pair of values at tap e.
+struct InputCols {
+    static constexpr bool kAsync = true;
+    const __nv_bfloat16* xb;
     int B;
-    __device__ uint4 operator()(int m, int k) const {
-        float v[8];
-        const int b = m >> 8, l = m & 255;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int e = k + i, kk = e >> 1, c = e & 1, j = l + kk - 2;
-            v[i] = (m < B * 256 && e < 10 && j >= 0 && j < 256) ? x[((size_t)b * 256 + j) * 2 + c] : 0.f;
-        }
-        return pack8(v);
+    __device__ const void* src(int m, int e) const {
+        return (m >> 8) < B ? xb + ((size_t)(m >> 8) * 260 + (m & 255) + e) * 2 : nullptr;
     }
 };
 
-// MN-major twin for the first layer's weight gradient; column 10 reads as 1
-struct InputIm2colT {
-    const float* x;
-    int B;
-    __device__ uint4 operator()(int r, int m) const {
-        float v[8];
-        const int b = r >> 8, l = r & 255;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int e = m + i, kk = e >> 1, c = e & 1, j = l + kk - 2;
-            float val = 0.f;
-            if (r < B * 256) {
-                if (e < 10) val = (j >= 0 && j < 256) ? x[((size_t)b * 256 + j) * 2 + c] : 0.f;
-                else if (e == 10) val = 1.f;
-            }
-            v[i] = val;
-        }
-        return pack8(v);
-    }
-};
-
-// col2im as a gather, for the input gradient of a convolution with output gradient dz [B][Lo][64]:
-// row m = b * L + i (input position), column k = kk * 64 + o ->
-// dz[b][(i + 2 - kk) / s][o] when s divides i + 2 - kk and the quotient is inside [0, Lo)
-struct Col2im {
+// The input gradient of such a convolution from its output gradient dz [B][Lo][64], Lo = 2^log_lo: the
+// input positions 2 p + PAR of a sample get dz[p + 1 - j] through tap kk = 2 j + PAR, j = 0 .. 2 (PAR 0) or
+// 0 .. 1 (PAR 1), so each parity is a product over its own taps and no zeros are multiplied:
+// row m = b * Lo + p, column k = j * 64 + o   (K-major A)
+template <int PAR>
+struct ConvGrad {
+    static constexpr bool kAsync = true;
     const __nv_bfloat16* dz;
-    int B, L, Lo, s;
-    __device__ uint4 operator()(int m, int k) const {
-        if (m >= B * L || k >= 5 * 64) return make_uint4(0, 0, 0, 0);
-        const int b = m / L, i = m - b * L, kk = k >> 6, o = k & 63;
-        const int num = i + 2 - kk;
-        if (num < 0 || num % s) return make_uint4(0, 0, 0, 0);
-        const int l = num / s;
-        if (l >= Lo) return make_uint4(0, 0, 0, 0);
-        return *reinterpret_cast<const uint4*>(dz + ((size_t)b * Lo + l) * 64 + o);
+    int B, log_lo;
+    __device__ const void* base() const { return dz; }
+    __device__ const void* src(int m, int k) const {
+        const int b = m >> log_lo, l = (m & ((1 << log_lo) - 1)) + 1 - (k >> 6);
+        if (b >= B || k >= (3 - PAR) * 64 || l < 0 || l >= (1 << log_lo)) return nullptr;
+        return dz + (((size_t)b << log_lo) + l) * 64 + (k & 63);
     }
 };
 
-// a convolution weight W [(kk * 64 + c)][o] read as the K-major B of the input gradient:
-// stored row n = c, column k = kk * 64 + o
+// a convolution weight W [(kk * 64 + c)][o] read as the K-major B of that product:
+// stored row n = c, column k = j * 64 + o, kk = 2 j + PAR
+template <int PAR>
 struct ConvWT {
+    static constexpr bool kAsync = true;
     const __nv_bfloat16* w;
-    __device__ uint4 operator()(int n, int k) const {
-        if (n >= 64 || k >= 5 * 64) return make_uint4(0, 0, 0, 0);
-        const int kk = k >> 6, o = k & 63;
-        return *reinterpret_cast<const uint4*>(w + ((size_t)kk * 64 + n) * 64 + o);
+    __device__ const void* base() const { return w; }
+    __device__ const void* src(int n, int k) const {
+        if (n >= 64 || k >= (3 - PAR) * 64) return nullptr;
+        return w + ((size_t)(2 * (k >> 6) + PAR) * 64 + n) * 64 + (k & 63);
     }
 };
 
