@@ -3,6 +3,7 @@
 
 #include "forward.cuh"
 #include "forward_launch.cuh"
+#include "refine.cuh"
 
 namespace sblm {
 
@@ -102,15 +103,22 @@ constexpr double kResolveCubic = 1e-6;
 static __device__ __noinline__ double resolve_fp64(const cx<float>* z32, uint32_t why, const Cand* kk,
                                                    double te, double fe, double we, double* A_row,
                                                    uint8_t* f_row, int e, bool chi2) {
-    cx<double> zz[5];
+    const cx<double> zeta = zeta64(*kk, te);
+    double A;
+    uint8_t flag = 0;
+    if (!resolve_thread(z32, zeta, kk->d, kk->q, &A)) {
+        cx<double> zz[5];
 #pragma unroll
-    for (int i = 0; i < 5; ++i) zz[i] = mk<double>(z32[i].re, z32[i].im);
-    bool w2 = true;
-    const EpochOut<double> o2 = solve_epoch<double>(zeta64(*kk, te), kk->d, kk->q, zz, w2, nullptr, kResolveCubic);
-    if (A_row) A_row[e] = o2.A;
-    if (f_row) f_row[e] = (uint8_t)(o2.flag | FLAG_FP64 | why);
+        for (int i = 0; i < 5; ++i) zz[i] = mk<double>(z32[i].re, z32[i].im);
+        bool w2 = true;
+        const EpochOut<double> o2 = solve_epoch<double>(zeta, kk->d, kk->q, zz, w2, nullptr, kResolveCubic);
+        A = o2.A;
+        flag = o2.flag;
+    }
+    if (A_row) A_row[e] = A;
+    if (f_row) f_row[e] = (uint8_t)(flag | FLAG_FP64 | why);
     if (!chi2) return 0.0;
-    const double r = (fe - o2.A) * we;
+    const double r = (fe - A) * we;
     return r * r;
 }
 

@@ -156,9 +156,9 @@ constexpr int kResolveLanes = 5, kResolvePerWarp = 6;
 // smallest gap between them goes to the general solver (0.02% of the re-solved epochs of the sweep)
 constexpr float kTightRoots = 3e-3f;
 // an epoch with an image at |det J| below this goes to the general solver: A's rounding error there,
-// about 2^-53 / (det J)^2 relative, is above 1e-10, and which way it falls is that solver's (0.1% of
-// the re-solved epochs)
-constexpr float kFoldDet = 1e-3f;
+// about 2^-53 / (det J)^2 relative, reaches 1e-9, and which way it falls is that solver's (0.03% of the
+// re-solved epochs; at 1e-3 four times as many, each of which holds up a small call by 100 us)
+constexpr float kFoldDet = 5e-4f;
 // least relative lens-equation residual at which a root of the quintic counts as spurious: computed
 // in FP32 after the images were divided out, and in FP64 after the FP64 root iteration
 constexpr float kSpuriousResidual32 = 1e-4f;
@@ -205,11 +205,10 @@ __device__ __forceinline__ double image_sum(const Refined& f, int base) {
     return sum;
 }
 
-// The two roots of the quintic that remain once three images are divided out (their sum and product
-// from its coefficients and the images), lane r taking one of them: whether that root is far from
-// solving the lens equation.
-__device__ __forceinline__ bool remaining_root_spurious(const Refined& f, cx<double> zeta, double d, double q, int base,
-                                                        int r) {
+// The two roots of the quintic that remain once three images (sum `zs`, product `zp`) are divided out,
+// from its coefficients; `which` selects one: whether that root is far from solving the lens equation.
+__device__ __forceinline__ bool remaining_root_spurious(cx<double> zs, cx<double> zp, cx<double> zeta, double d,
+                                                        double q, int which) {
     const cx<double> s = conj(zeta);
     const double m = 1.0 + q;
     const cx<double> n1 = mk<double>(fma(-d, s.re, m), -d * s.im), k2 = mk<double>(s.re - d, s.im);
@@ -218,15 +217,8 @@ __device__ __forceinline__ bool remaining_root_spurious(const Refined& f, cx<dou
     const cx<double> c4 = s * k1 + n1 * k2 - zeta * c5 - k2 - q * s;
     const double rc = rcp_cubic(norm2(c5));
     const cx<double> ic5 = mk<double>(c5.re * rc, -c5.im * rc);
-    cx<double> h = -(c4 * ic5), prod = mk<double>(1.0, 0.0);
-    const cx<double> zs = f.image ? f.z : mk<double>(0.0, 0.0), zp = f.image ? f.z : prod;
-#pragma unroll
-    for (int j = 0; j < 5; ++j) {
-        h = h - shfl(zs, base + j);
-        prod = prod * shfl(zp, base + j);
-    }
-    h = 0.5 * h;
-    const cx<double> den = c5 * prod;  // the quintic's roots multiply to d^2 zeta / c5
+    const cx<double> h = -0.5 * (c4 * ic5 + zs);
+    const cx<double> den = c5 * zp;  // the quintic's roots multiply to d^2 zeta / c5
     const double rd = rcp_cubic(norm2(den)) * (d * d);
     const cx<double> P = zeta * mk<double>(den.re * rd, -den.im * rd);
     const cx<double> D = h * h - P;
@@ -235,7 +227,7 @@ __device__ __forceinline__ bool remaining_root_spurious(const Refined& f, cx<dou
     const float mod = sqrt_(norm2(Df));
     float sr = sqrt_(fmax(0.5f * (mod + Df.re), 0.f)), si = sqrt_(fmax(0.5f * (mod - Df.re), 0.f));
     if (Df.im < 0.f) si = -si;
-    if (r & 1) {
+    if (which & 1) {
         sr = -sr;
         si = -si;
     }
@@ -329,7 +321,14 @@ __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<doubl
     bool done = open && count == 5 && parity == -1;
     const bool three = open && count == 3 && parity == -1;
     if (__any_sync(0xffffffffu, three)) {
-        const bool sp = remaining_root_spurious(f, zeta, d, q, base, r);
+        cx<double> zs = mk<double>(0.0, 0.0), zp = mk<double>(1.0, 0.0);
+        const cx<double> mine_s = f.image ? f.z : zs, mine_p = f.image ? f.z : zp;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            zs = zs + shfl(mine_s, base + j);
+            zp = zp * shfl(mine_p, base + j);
+        }
+        const bool sp = remaining_root_spurious(zs, zp, zeta, d, q, r);
         const unsigned b = __ballot_sync(0xffffffffu, sp) >> base & 3u;
         done = done || (three && b == 3u);
     }
@@ -380,6 +379,56 @@ __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<doubl
     }
     *A = sum;
     return done && !fold;
+}
+
+// resolve_group's first stage by one thread, its roots one after the other: for callers that re-solve a
+// few epochs each in its own thread. False where it is open: the general solver's.
+__device__ __forceinline__ bool resolve_thread(const cx<float>* z32, cx<double> zeta, double d, double q, double* A) {
+    const cx<float> zetaf = mk<float>((float)zeta.re, (float)zeta.im);
+    if (!refine_lens((float)d, (float)q) || !refine_source(zetaf, (float)d)) return false;
+    for (int i = 0; i < 5; ++i) {
+        const float az = sqrt_(norm2(z32[i]));
+        float num = 2.f * az, den = 1.f, gap = INFINITY;
+        for (int j = 0; j < 5; ++j) {
+            if (j == i) continue;
+            const float dd = sqrt_(norm2(z32[i] - z32[j]));
+            num *= az + sqrt_(norm2(z32[j]));
+            den *= dd;
+            gap = fmin(gap, dd);
+        }
+        if (!((kNoise * 1.1102230e-16f) * num <= kTightRoots * den * gap)) return false;
+    }
+    cx<float> zi[5], wi[5];  // the images found
+    int count = 0, parity = 0;
+    bool fold = false;
+    double sum = 0.0;
+    cx<double> zs = mk<double>(0.0, 0.0), zp = mk<double>(1.0, 0.0);
+    for (int i = 0; i < 5; ++i) {
+        cx<double> z, w;
+        start_from_fp32(z32[i], d, z, w);
+        const Refined f = refine_root(z, w, zeta, q, 8);
+        if (!f.image) continue;
+        const cx<float> zf = mk<float>((float)f.z.re, (float)f.z.im), wf = mk<float>((float)f.w.re, (float)f.w.im);
+        bool dup = false;
+        for (int j = 0; j < count; ++j)
+            dup = dup || (norm2(zi[j] - zf) <= 1e-11f * fmin(norm2(zi[j]), norm2(zf)) &&
+                          norm2(wi[j] - wf) <= 1e-11f * fmin(norm2(wi[j]), norm2(wf)));
+        if (dup) continue;
+        zi[count] = zf;
+        wi[count] = wf;
+        ++count;
+        parity += f.det < 0.0 ? -1 : 1;
+        const double a = fabs(f.det);
+        fold = fold || (float)a < kFoldDet;
+        sum += rcp_cubic(a);
+        zs = zs + f.z;
+        zp = zp * f.z;
+    }
+    *A = sum;
+    if (parity != -1 || fold) return false;
+    if (count == 5) return true;
+    return count == 3 && remaining_root_spurious(zs, zp, zeta, d, q, 0) &&
+           remaining_root_spurious(zs, zp, zeta, d, q, 1);
 }
 
 }  // namespace sblm
