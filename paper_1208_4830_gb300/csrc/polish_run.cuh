@@ -1,4 +1,9 @@
 // polish_run.cuh -- one thread's run of consecutive epochs of one candidate in the amoeba's objective.
+// A copy of the epoch loop apart from forward_run.cuh's: the compiler fuses the FP32 products here in
+// another way at each of the kernel's call sites, and any change of the loop moves MIXED chi^2 by 1e-7,
+// which a simplex amplifies. What bounds the amoeba is the chain of one chi^2 after the other; the FP64
+// re-solves in place were a third of it: 64 curves of 500 epochs, 200 evaluations, 35.2 ms with the general
+// solver for each, 23.8 ms with the epoch's roots refined first (resolve_thread).
 #pragma once
 
 #include "forward.cuh"
@@ -69,27 +74,6 @@ __device__ __forceinline__ Cand candidate(const double* __restrict__ src, const 
     sincos(a[3], &k.sa, &k.ca);
     k.d = a[4];
     k.q = exp10(a[5]);
-    return k;
-}
-
-// The candidate of a group of G threads (G a power of two; groups are aligned to G within the
-// warp, or span whole warps when G > 32), decoded once per warp-part by its first lane and
-// broadcast by shuffles: the decode's FP64 exp10, sincos and division run on the slow FP64 pipe.
-// Every lane of the warp must call it.
-template <bool FROM_GENES>
-__device__ __forceinline__ Cand group_candidate(const double* __restrict__ src, const Bounds& b, int c, bool valid,
-                                                int G) {
-    const int lane = threadIdx.x & 31;
-    const int src_lane = G < 32 ? (lane & ~(G - 1)) : 0;
-    Cand k{};
-    if (lane == src_lane && valid) k = candidate<FROM_GENES>(src, b, c);
-    k.t0 = __shfl_sync(0xffffffffu, k.t0, src_lane);
-    k.inv_tE = __shfl_sync(0xffffffffu, k.inv_tE, src_lane);
-    k.u0 = __shfl_sync(0xffffffffu, k.u0, src_lane);
-    k.sa = __shfl_sync(0xffffffffu, k.sa, src_lane);
-    k.ca = __shfl_sync(0xffffffffu, k.ca, src_lane);
-    k.d = __shfl_sync(0xffffffffu, k.d, src_lane);
-    k.q = __shfl_sync(0xffffffffu, k.q, src_lane);
     return k;
 }
 
@@ -230,16 +214,6 @@ __device__ __forceinline__ double eval_run(const Cand& k, bool valid, int c_tag,
         }
     }
     return chi;
-}
-
-// MIXED: sum of a candidate's term row over the lanes of its group of G threads (G a power of two
-// <= 32, groups aligned within the warp): lane g adds epochs g, g + G, ... in order, then a fixed
-// butterfly combines the lanes; every lane of the group gets the sum. All lanes of the warp call it.
-__device__ __forceinline__ double term_row_sum(const double* __restrict__ row, int n_ep, int g, int G, bool valid) {
-    double s = 0.0;
-    for (int e = g; valid && e < n_ep; e += G) s += row[e];
-    for (int off = G / 2; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    return s;
 }
 
 }  // namespace sblm

@@ -11,7 +11,8 @@
 // until the correction is below kRefineStep min(1, |det J|) of the distance to the nearer lens; the
 // Jacobian at the last point in FP64, advanced by that last correction to first order, gives det J.
 // 18 FP64 instructions per step and about 20 for the last one, against some 250 per root and sweep
-// of a root iteration in FP64.
+// of a root iteration in FP64. FP64 chi^2 of 4096 x 2000: 68.6 ms with the quintic solved in FP64, 8.2 ms so;
+// one event's curve of 400 epochs: 1186 us, 208 us.
 #pragma once
 
 #include "forward.cuh"
