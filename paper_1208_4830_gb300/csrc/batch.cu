@@ -297,18 +297,27 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
                 if constexpr (MODE != SBLM_FP32) {
                     // the block's queued epochs, in FP64 from the FP64 data, each term to its place
                     // in the candidate's term row; then each candidate's row summed in a fixed order
-                    resolve_queue(
-                        sink.queue, min(s_qcount, a.qcap), threadIdx.x >> 5, blockDim.x >> 5,
-                        [&](int cq) { return cand_blk[cq]; },
-                        [&](int, int e) {
-                            const int64_t ge = e_begin + e;
-                            return EpochData{a.t[ge], a.flux[ge], 1.0 / a.sigma[ge]};
-                        },
-                        [&](int cq, int e, double A, uint8_t flag, uint32_t why, double fe, double we) {
-                            double* A_rq = a.blend ? a.A_scr + ((size_t)blockIdx.x * n_pop + cq) * a.max_ep : nullptr;
-                            term_blk[(size_t)cq * a.max_ep + e] =
-                                store_resolved<MODE>(A, flag, why, fe, we, A_rq, nullptr, e);
-                        });
+                    const unsigned n_q = min(s_qcount, a.qcap);
+                    const auto cand_of = [&](int cq) { return cand_blk[cq]; };
+                    const auto data_of = [&](int, int e) {
+                        const int64_t ge = e_begin + e;
+                        return EpochData{a.t[ge], a.flux[ge], 1.0 / a.sigma[ge]};
+                    };
+                    const auto store = [&](int cq, int e, double A, uint8_t flag, uint32_t why, double fe, double we) {
+                        double* A_rq = a.blend ? a.A_scr + ((size_t)blockIdx.x * n_pop + cq) * a.max_ep : nullptr;
+                        term_blk[(size_t)cq * a.max_ep + e] =
+                            store_resolved<MODE>(A, flag, why, fe, we, A_rq, nullptr, e);
+                    };
+                    // MIXED queues longer than the block has threads: a lane per epoch, all by the general
+                    // solver. Populations that have gathered at a caustic queue thousands of epochs, so many
+                    // of them for the general solver that nearly every warp of six waits for one such lane,
+                    // where 32 lanes share its passes (152 curves of 500 epochs, 1024 x 300 generations:
+                    // 10.4 s, 12.4 s with six epochs per warp throughout); the short queues of the first
+                    // generations are bound by one epoch's latency, and the groups' is a tenth.
+                    if (MODE == SBLM_MIXED && n_q > blockDim.x)
+                        resolve_queue_lanes(sink.queue, n_q, threadIdx.x, blockDim.x, cand_of, data_of, store);
+                    else
+                        resolve_queue(sink.queue, n_q, threadIdx.x >> 5, blockDim.x >> 5, cand_of, data_of, store);
                     __syncthreads();
                     for (int base = 0; base < n_pop; base += per_pass) {
                         const int cand = base + group;

@@ -161,6 +161,20 @@ __device__ __forceinline__ void resolve_queue(const Deferred* __restrict__ queue
     }
 }
 
+// The same with the general solver, a lane per epoch: lane `first` takes epochs first, first + step, ...
+template <class CandFn, class DataFn, class StoreFn>
+__device__ __forceinline__ void resolve_queue_lanes(const Deferred* __restrict__ queue, unsigned n, unsigned first,
+                                                    unsigned step, CandFn cand, DataFn data, StoreFn store) {
+    for (unsigned i = first; i < n; i += step) {
+        const Deferred& q = queue[i];
+        const Cand k = cand(q.c);
+        const EpochData ed = data(q.c, q.e);
+        uint8_t flag;
+        const double A = solve_general(q.z, &k, ed.t, &flag);
+        store(q.c, q.e, A, flag, q.why, ed.flux, ed.w);
+    }
+}
+
 // The thread's epochs [e0, e1) of candidate k (all lanes of a warp run `seg` iterations so that
 // queue slots can be reserved warp-wide). Writes A and flags when the row pointers are given.
 // FP32: returns the thread's chi^2 over its epochs, accumulated in FP64 in epoch order. MIXED and
