@@ -483,27 +483,6 @@ __global__ void adam_scalars_kernel(AdamArgs ad, const int64_t* ctr, double* out
     if (threadIdx.x < 3) out[threadIdx.x] = adam_scalar(ad, ctr[0] + 1, threadIdx.x);
 }
 
-// 1/x and sqrt(x) of positive doubles to a few 2^-53: a hardware approximation and Newton steps (the
-// library's division and square root are some 70 instructions of the FP64 pipe, which bounded this
-// kernel with the bias corrections' powers in every block: 49 us for 326,156 parameters, 32 us with both
-// taken out); sqrt(0) = 0
-__device__ __forceinline__ double reciprocal(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-__device__ __forceinline__ double square_root(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    // y <- y + y e / 2 + 3 y e^2 / 8, e = 1 - x y^2, then one correction of s = x y
-    const double e = fma(-x * y, y, 1.0);
-    y = fma(y * e, fma(0.375, e, 0.5), y);
-    const double s = x * y;
-    const double t = fma(0.5 * y, fma(-s, s, x), s);
-    return x > 0.0 && isfinite(t) ? t : sqrt(x);
-}
-
 // gradient = sum of the partials in split order (or grad_in); optional AdamW step and BF16 copies
 __global__ void update_kernel(PartTab tab, const float* grad_in, float* grad_out, AdamArgs ad, float* w,
                               __nv_bfloat16* wb, __nv_bfloat16* wbt) {
@@ -544,7 +523,7 @@ __global__ void update_kernel(PartTab tab, const float* grad_in, float* grad_out
         const double v = ad.b2 * (double)ad.v[idx] + (1.0 - ad.b2) * (double)g * g;
         const double mh = m * s_sc[1];
         const double vh = v * s_sc[2];
-        wd = wd - lr * mh * reciprocal(square_root(vh) + ad.eps);
+        wd = wd - lr * mh / (sqrt(vh) + ad.eps);
         ad.m[idx] = (float)m;
         ad.v[idx] = (float)v;
         wv = (float)wd;
