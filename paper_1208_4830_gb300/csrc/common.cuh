@@ -41,9 +41,10 @@ __device__ __forceinline__ float rcp(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
-// FP64: hardware reciprocal approximation (relative error ~1e-6 on sm_103a) and two Newton
-// steps r <- r (2 - x r), which square the error each time; the IEEE division is an order of
-// magnitude dearer on the FP64 pipe. Zero, infinite and NaN inputs keep the approximation's
+// FP64: hardware reciprocal approximation (relative error about 2^-20) and two Newton-Raphson steps
+// r <- r (2 - x r), which square the error each time (2^-40, 2^-80) and leave the roundings of the last one:
+// within 2^-52 of 1/x for normal x with a normal reciprocal (tests/test_gpu_reciprocal.py). The IEEE division is
+// an order of magnitude dearer on the FP64 pipe. Zero, infinite and NaN inputs keep the approximation's
 // value (inf, 0, NaN).
 __device__ __forceinline__ double rcp(double x) {
     double r;
@@ -54,6 +55,16 @@ __device__ __forceinline__ double rcp(double x) {
     }
     return r;
 }
+// One Newton-Raphson step of the reciprocal in residual form, r <- r + r (1 - x r): the residual is exact to
+// its own rounding, so the step rounds once. rcp_start: the approximation and one step (2^-40); rcp_normal: two,
+// within 2^-53 (1 + 2^-26) of 1/x for normal x with a normal reciprocal; zero and infinity give NaN.
+__device__ __forceinline__ double rcp_step(double x, double r) { return fma(r, fma(-x, r, 1.0), r); }
+__device__ __forceinline__ double rcp_start(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return rcp_step(x, r);
+}
+__device__ __forceinline__ double rcp_normal(double x) { return rcp_step(x, rcp_start(x)); }
 
 __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
 __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }

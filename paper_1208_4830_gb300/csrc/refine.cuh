@@ -10,9 +10,9 @@
 // shrinks the error by the FP32 Jacobian's relative error, about 2e-7 / |det J|, and quadratically)
 // until the correction is below kRefineStep min(1, |det J|) of the distance to the nearer lens; the
 // Jacobian at the last point in FP64, advanced by that last correction to first order, gives det J.
-// 18 FP64 instructions per step and about 20 for the last one, against some 250 per root and sweep
-// of a root iteration in FP64. FP64 chi^2 of 4096 x 2000: 68.6 ms with the quintic solved in FP64, 8.2 ms so;
-// one event's curve of 400 epochs: 1186 us, 208 us.
+// 16 FP64 instructions for the first step, 20 for each further one and about 20 for the last one's Jacobian,
+// against some 250 per root and sweep of a root iteration in FP64. FP64 chi^2 of 4096 x 2000: 68.6 ms with the
+// quintic solved in FP64, 8.4 ms so; one event's curve of 400 epochs: 1186 us, 215 us.
 #pragma once
 
 #include "forward.cuh"
@@ -36,15 +36,6 @@ __device__ __forceinline__ bool refine_source(cx<float> zeta, float d) {
            norm2(mk<float>(zeta.re - d, zeta.im)) >= 1e-12f;
 }
 
-// reciprocal of a positive double: hardware approximation (relative error below 2^-20) and one step
-// r (1 + e + e^2), e = 1 - x r, which leaves e^3
-__device__ __forceinline__ double rcp_cubic(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // one root in FP64: its position from the primary (z) and from the secondary (w = z - d), both
 // advanced by every correction so that the one that is small keeps its relative precision
 struct Refined {
@@ -63,7 +54,12 @@ __device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<do
 #pragma unroll 1
     for (int it = 0;; ++it) {
         const double n1 = norm2(z), n2 = norm2(w);
-        const double r1 = rcp_cubic(n1), r2 = rcp_cubic(n2);
+        // the first correction is one of FP32's errors, and one Newton step gives its residual 2^-40
+        double r1 = rcp_start(n1), r2 = rcp_start(n2);
+        if (it > 0) {
+            r1 = rcp_step(n1, r1);
+            r2 = rcp_step(n2, r2);
+        }
         const double qr2 = q * r2;
         // u = 1/conj(z) = z r1, v = 1/(d - conj(z)) = -w r2; f = z - u + q v - zeta
         cx<double> f;
@@ -83,7 +79,7 @@ __device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<do
         const float n1f = (float)n1, n2f = (float)n2;
         const float scale = sqrt_(n1f) + sqrt_(r1f) + qf * sqrt_(r2f) + zeta_abs;
         const float lim = fmax(kRefineStep * fmin(ad, 1.f) * sqrt_(fmin(n1f, n2f)), 1e-15f * scale * rad);
-        const bool last = d2 <= lim * lim;
+        const bool last = it > 0 && d2 <= lim * lim;
         if (last) {
             // K in FP64 at (z, w), and det J advanced by delta: dK = 2 conj(delta) (q v^3 - u^3)
             const double uu = r1 * r1, vv = qr2 * r2;
@@ -141,7 +137,7 @@ __device__ __forceinline__ bool refine_images(const Root<float> rp[5], unsigned 
         const cx<float> moved = mk<float>((float)(f.w.re - w.re), (float)(f.w.im - w.im));
         ok = ok && f.image && norm2(moved) <= 1e-6f * gap2;
         const double a = fabs(f.det);
-        sum += rcp_cubic(a);
+        sum += rcp_normal(a);
         parity += f.det < 0.0 ? -1 : 1;
     }
     *A = sum;
@@ -199,7 +195,7 @@ __device__ __forceinline__ void count_images(const Refined& f, int base, int* co
 
 // sum over the group's images of 1/|det J|, in root order, in every lane of the group
 __device__ __forceinline__ double image_sum(const Refined& f, int base) {
-    const double a = f.image ? rcp_cubic(fabs(f.det)) : 0.0;
+    const double a = f.image ? rcp_normal(fabs(f.det)) : 0.0;
     double sum = 0.0;
 #pragma unroll
     for (int s = 0; s < 5; ++s) sum += __shfl_sync(0xffffffffu, a, base + s);
@@ -216,11 +212,11 @@ __device__ __forceinline__ bool remaining_root_spurious(cx<double> zs, cx<double
     const cx<double> k1 = mk<double>(fma(d, d, n1.re), n1.im);
     const cx<double> c5 = s * k2;
     const cx<double> c4 = s * k1 + n1 * k2 - zeta * c5 - k2 - q * s;
-    const double rc = rcp_cubic(norm2(c5));
+    const double rc = rcp_normal(norm2(c5));
     const cx<double> ic5 = mk<double>(c5.re * rc, -c5.im * rc);
     const cx<double> h = -0.5 * (c4 * ic5 + zs);
     const cx<double> den = c5 * zp;  // the quintic's roots multiply to d^2 zeta / c5
-    const double rd = rcp_cubic(norm2(den)) * (d * d);
+    const double rd = rcp_normal(norm2(den)) * (d * d);
     const cx<double> P = zeta * mk<double>(den.re * rd, -den.im * rd);
     const cx<double> D = h * h - P;
     // the square root in FP32: the two roots to FP32 accuracy relative to their distance
@@ -421,7 +417,7 @@ __device__ __forceinline__ bool resolve_thread(const cx<float>* z32, cx<double> 
         parity += f.det < 0.0 ? -1 : 1;
         const double a = fabs(f.det);
         fold = fold || (float)a < kFoldDet;
-        sum += rcp_cubic(a);
+        sum += rcp_normal(a);
         zs = zs + f.z;
         zp = zp * f.z;
     }
