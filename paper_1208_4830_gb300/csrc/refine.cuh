@@ -287,6 +287,9 @@ static __device__ __noinline__ cx<double> lane_aberth(cx<double> z, bool move, c
 __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<double> zeta, double d, double q, double* A) {
     const int lane = threadIdx.x & 31;
     const int grp = lane / kResolveLanes, base = grp * kResolveLanes, r = lane - base;
+    const cx<float> zetaf = mk<float>((float)zeta.re, (float)zeta.im);
+    const bool in_range = valid && refine_lens((float)d, (float)q) && refine_source(zetaf, (float)d);
+    if (!__any_sync(0xffffffffu, in_range)) return false;
     // the smallest gap between this root and the others, and the quintic's rounding noise at it,
     // kNoise eps prod (|z| + |z_j|) / prod |z - z_j| (j = i included above)
     const float az = sqrt_(norm2(zf));
@@ -300,9 +303,8 @@ __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<doubl
         gap = fmin(gap, dd);
     }
     const bool loose = (kNoise * 1.1102230e-16f) * num <= kTightRoots * den * gap;  // false for NaN
-    const cx<float> zetaf = mk<float>((float)zeta.re, (float)zeta.im);
     const unsigned loose_lanes = __ballot_sync(0xffffffffu, loose) >> base & 31u;
-    const bool open = valid && loose_lanes == 31u && refine_lens((float)d, (float)q) && refine_source(zetaf, (float)d);
+    const bool open = in_range && loose_lanes == 31u;
     if (!__any_sync(0xffffffffu, open)) return false;
     cx<double> z, w;
     start_from_fp32(zf, d, z, w);
