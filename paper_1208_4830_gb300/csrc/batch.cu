@@ -314,7 +314,9 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
                     // where 32 lanes share its passes (152 curves of 500 epochs, 1024 x 300 generations:
                     // 10.4 s, 12.4 s with six epochs per warp throughout); the short queues of the first
                     // generations are bound by one epoch's latency, and the groups' is a tenth.
-                    if (MODE == SBLM_MIXED && n_q > blockDim.x)
+                    // The same in either mode when more epochs deferred than the queue holds: which of them it
+                    // holds is a race, and the others went to the general solver in place.
+                    if ((MODE == SBLM_MIXED && n_q > blockDim.x) || s_qcount > a.qcap)
                         resolve_queue_lanes(sink.queue, n_q, threadIdx.x, blockDim.x, cand_of, data_of, store);
                     else
                         resolve_queue(sink.queue, n_q, threadIdx.x >> 5, blockDim.x >> 5, cand_of, data_of, store);
@@ -589,11 +591,8 @@ sblm_status prepare(const double* t, const double* flux, const double* sigma, co
     SBLM_TRY(is_device_pointer(sigma, &d3));
     if (!d1 && !d2 && !d3) SBLM_TRY(check_lightcurve_host(t, flux, sigma, (int)total));
     // per block: room for a quarter of a generation's epochs (a population gathered on a
-    // caustic-crossing model defers many); epochs past this are re-solved in place, one divergent
-    // lane at a time, so the size is a speed choice only
-    // per block: room for a quarter of a generation's epochs (a population gathered on a
-    // caustic-crossing model defers many), within 2^26 entries (~3 GB) over all blocks; epochs past
-    // this are re-solved in place, one divergent lane at a time, so the size is a speed choice only
+    // caustic-crossing model defers many), within 2^26 entries (~3 GB) over all blocks; when more defer,
+    // all of them take the general solver, those past this in place, one divergent lane at a time
     const unsigned qcap =
         mode != SBLM_FP32
             ? (unsigned)std::max<long>(4096, std::min<long>((long)c.n_pop * max_ep / 4, (1L << 26) / blocks))

@@ -41,18 +41,24 @@ __global__ void __launch_bounds__(kResolveBlock) resolve_kernel(const Cand* __re
                                                                 const unsigned* __restrict__ count, unsigned cap,
                                                                 double* __restrict__ A_out, uint8_t* __restrict__ flags,
                                                                 double* __restrict__ term) {
-    const unsigned n = min(*count, cap);
-    resolve_queue(
-        queue, n, (threadIdx.x >> 5) * gridDim.x + blockIdx.x, gridDim.x * (kResolveBlock / 32),
-        [&](int c) { return cands[c]; },
-        [&](int, int e) {
-            return EpochData{t[e], CHI2 ? flux[e] : 0.0, CHI2 ? 1.0 / sigma[e] : 0.0};
-        },
-        [&](int c, int e, double A, uint8_t flag, uint32_t why, double fe, double we) {
-            const double tm = store_resolved<MODE>(A, flag, why, fe, we, A_out ? A_out + (size_t)c * n_ep : nullptr,
-                                                   flags ? flags + (size_t)c * n_ep : nullptr, e);
-            if (CHI2) term[(size_t)c * n_ep + e] = tm;
-        });
+    const unsigned total = *count, n = min(total, cap);
+    const auto cand_of = [&](int c) { return cands[c]; };
+    const auto data_of = [&](int, int e) {
+        return EpochData{t[e], CHI2 ? flux[e] : 0.0, CHI2 ? 1.0 / sigma[e] : 0.0};
+    };
+    const auto store = [&](int c, int e, double A, uint8_t flag, uint32_t why, double fe, double we) {
+        const double tm = store_resolved<MODE>(A, flag, why, fe, we, A_out ? A_out + (size_t)c * n_ep : nullptr,
+                                               flags ? flags + (size_t)c * n_ep : nullptr, e);
+        if (CHI2) term[(size_t)c * n_ep + e] = tm;
+    };
+    // more epochs deferred than the queue holds: which of them it holds is a race, and the others went to the
+    // general solver in place, so these go to it too
+    if (total > cap)
+        resolve_queue_lanes(queue, n, blockIdx.x * kResolveBlock + threadIdx.x, gridDim.x * kResolveBlock, cand_of,
+                            data_of, store);
+    else
+        resolve_queue(queue, n, (threadIdx.x >> 5) * gridDim.x + blockIdx.x, gridDim.x * (kResolveBlock / 32), cand_of,
+                      data_of, store);
 }
 
 // MIXED and FP64, third pass: chi^2 of candidate (warp) c as the sum of its term row in a fixed order
@@ -232,11 +238,12 @@ MixedLayout mixed_layout(int mode, int n_cand, int n_ep, bool chi2) {
     MixedLayout l;
     if (mode == SBLM_FP32 || n_cand <= 0 || n_ep <= 0) return l;
     if (mode == SBLM_FP64) n_cand = fp64_chunk(n_cand, n_ep);
-    // a queue entry for one epoch in 32 (0.35% of the sweep's epochs defer in MIXED, 2.6% of those of
-    // the trajectories aimed at caustics), for FP64's wider triggers one in 8; at least 4096 and at most
-    // 2^24 entries (0.9 GB)
+    // MIXED: a queue entry for one epoch in 32 (0.35% of the sweep's epochs defer, 2.6% of those of the
+    // trajectories aimed at caustics). FP64: one for every epoch of a chunk, so that only a lightcurve beyond
+    // 2^24 epochs can overflow it: a lens outside the refined range defers all of them, and the others would
+    // lose their places to it. At least 4096 and at most 2^24 entries (0.9 GB).
     const long n = (long)n_cand * n_ep;
-    l.queue_cap = (unsigned)std::min<long>(std::max<long>(n / (mode == SBLM_FP64 ? 8 : 32), 4096), 1L << 24);
+    l.queue_cap = (unsigned)std::min<long>(std::max<long>(n / (mode == SBLM_FP64 ? 1 : 32), 4096), 1L << 24);
     auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
     l.off_count = up(sizeof(Deferred) * (size_t)l.queue_cap);
     l.off_cand = up(l.off_count + sizeof(unsigned));

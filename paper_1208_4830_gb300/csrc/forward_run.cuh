@@ -120,8 +120,9 @@ __device__ __forceinline__ double store_resolved(double A, uint8_t flag, uint32_
 }
 
 // Where MIXED and FP64 work goes. Epochs to re-solve in FP64 are appended to `queue` (slots taken
-// with one atomic per warp, so that a later pass re-solves them side by side; an epoch that finds
-// the queue full is re-solved in place, so the capacity is a speed choice only). Every epoch's chi^2
+// with one atomic per warp, so that a later pass re-solves them side by side). An epoch that finds
+// the queue full takes the general solver in place; the pass over the queue then sends the queued
+// ones to it too, so that an epoch's result does not depend on whether it found a place. Every epoch's chi^2
 // term is stored in the candidate's row of the dense term array (the others here, the re-solved ones
 // by the re-solve, wherever it runs), and the row is summed afterwards in a fixed order: the chi^2
 // does not depend on the order in which the queue filled. `term_row` is the candidate's row
