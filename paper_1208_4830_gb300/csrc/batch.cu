@@ -51,7 +51,8 @@ struct BatchArgs {
     uint64_t* keys;    // per block: n_pop x 6
     Deferred* queue;   // MIXED and FP64, per block: qcap entries
     unsigned qcap;
-    double* term;      // MIXED and FP64, per block: n_pop x max_ep chi^2 terms (row per candidate)
+    int rows;          // candidates evaluated between two passes over the queue
+    double* term;      // MIXED and FP64, per block: rows x max_ep chi^2 terms (row per candidate)
     Cand* cands;       // per block: n_pop decoded candidates of the population being evaluated
     unsigned* next;    // work counter
     double* best_theta;
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
         sink.queue_count = &s_qcount;
         sink.queue_cap = a.qcap;
     }
-    double* const term_blk = MODE != SBLM_FP32 ? a.term + (size_t)blockIdx.x * n_pop * a.max_ep : nullptr;
+    double* const term_blk = MODE != SBLM_FP32 ? a.term + (size_t)blockIdx.x * a.rows * a.max_ep : nullptr;
     Cand* const cand_blk = a.cands + (size_t)blockIdx.x * n_pop;
     const int m = n_pop * n_par;
     double* const Pi = a.P + (size_t)blockIdx.x * n_isl * 2 * m;  // island i: rows Pi + i 2m (two buffers)
@@ -281,53 +282,59 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
                 }
                 decode_candidates<true>(Pc, a.b, 0, n_pop, n_pop, cand_blk, nullptr);
                 __syncthreads();
-                for (int base = 0; base < n_pop; base += per_pass) {
-                    const int cand = base + group;
-                    const bool valid = cand < n_pop;
-                    const Cand k = cand_blk[min(cand, n_pop - 1)];
-                    double* A_row =
-                        (a.blend && valid) ? a.A_scr + ((size_t)blockIdx.x * n_pop + cand) * a.max_ep : nullptr;
-                    double* term_row = (MODE != SBLM_FP32 && valid) ? term_blk + (size_t)cand * a.max_ep : nullptr;
-                    double chi = eval_run<MODE, true, true>(k, valid, cand, e0, e1, seg, view, A_row, nullptr, sink,
-                                                            term_row);
-                    for (int off = G / 2; off > 0; off >>= 1) chi += __shfl_xor_sync(0xffffffffu, chi, off);
-                    if (g == 0 && valid) s_chi[cand] = chi;
-                }
-                __syncthreads();
-                if constexpr (MODE != SBLM_FP32) {
-                    // the block's queued epochs, in FP64 from the FP64 data, each term to its place
-                    // in the candidate's term row; then each candidate's row summed in a fixed order
-                    const unsigned n_q = min(s_qcount, a.qcap);
-                    const auto cand_of = [&](int cq) { return cand_blk[cq]; };
-                    const auto data_of = [&](int, int e) {
-                        const int64_t ge = e_begin + e;
-                        return EpochData{a.t[ge], a.flux[ge], 1.0 / a.sigma[ge]};
-                    };
-                    const auto store = [&](int cq, int e, double A, uint8_t flag, uint32_t why, double fe, double we) {
-                        double* A_rq = a.blend ? a.A_scr + ((size_t)blockIdx.x * n_pop + cq) * a.max_ep : nullptr;
-                        term_blk[(size_t)cq * a.max_ep + e] =
-                            store_resolved<MODE>(A, flag, why, fe, we, A_rq, nullptr, e);
-                    };
-                    // MIXED queues longer than the block has threads: a lane per epoch, all by the general
-                    // solver. Populations that have gathered at a caustic queue thousands of epochs, so many
-                    // of them for the general solver that nearly every warp of six waits for one such lane,
-                    // where 32 lanes share its passes (152 curves of 500 epochs, 1024 x 300 generations:
-                    // 10.4 s, 12.4 s with six epochs per warp throughout); the short queues of the first
-                    // generations are bound by one epoch's latency, and the groups' is a tenth.
-                    // The same in either mode when more epochs deferred than the queue holds: which of them it
-                    // holds is a race, and the others went to the general solver in place.
-                    if ((MODE == SBLM_MIXED && n_q > blockDim.x) || s_qcount > a.qcap)
-                        resolve_queue_lanes(sink.queue, n_q, threadIdx.x, blockDim.x, cand_of, data_of, store);
-                    else
-                        resolve_queue(sink.queue, n_q, threadIdx.x >> 5, blockDim.x >> 5, cand_of, data_of, store);
-                    __syncthreads();
-                    for (int base = 0; base < n_pop; base += per_pass) {
+                for (int r0 = 0; r0 < n_pop; r0 += a.rows) {
+                    const int r1 = min(n_pop, r0 + a.rows);
+                    for (int base = r0; base < r1; base += per_pass) {
                         const int cand = base + group;
-                        const double* row = term_blk + (size_t)min(cand, n_pop - 1) * a.max_ep;
-                        const double chi = term_row_sum(row, n_ep, g, G, cand < n_pop);
-                        if (g == 0 && cand < n_pop) s_chi[cand] = chi;
+                        const bool valid = cand < r1;
+                        const Cand k = cand_blk[min(cand, n_pop - 1)];
+                        double* A_row =
+                            (a.blend && valid) ? a.A_scr + ((size_t)blockIdx.x * n_pop + cand) * a.max_ep : nullptr;
+                        double* term_row =
+                            (MODE != SBLM_FP32 && valid) ? term_blk + (size_t)(cand - r0) * a.max_ep : nullptr;
+                        double chi = eval_run<MODE, true, true>(k, valid, cand, e0, e1, seg, view, A_row, nullptr, sink,
+                                                                term_row);
+                        for (int off = G / 2; off > 0; off >>= 1) chi += __shfl_xor_sync(0xffffffffu, chi, off);
+                        if (g == 0 && valid) s_chi[cand] = chi;
                     }
                     __syncthreads();
+                    if constexpr (MODE != SBLM_FP32) {
+                        // the block's queued epochs, in FP64 from the FP64 data, each term to its place
+                        // in the candidate's term row; then each candidate's row summed in a fixed order
+                        const unsigned n_q = min(s_qcount, a.qcap);
+                        const auto cand_of = [&](int cq) { return cand_blk[cq]; };
+                        const auto data_of = [&](int, int e) {
+                            const int64_t ge = e_begin + e;
+                            return EpochData{a.t[ge], a.flux[ge], 1.0 / a.sigma[ge]};
+                        };
+                        const auto store = [&](int cq, int e, double A, uint8_t flag, uint32_t why, double fe,
+                                               double we) {
+                            double* A_rq = a.blend ? a.A_scr + ((size_t)blockIdx.x * n_pop + cq) * a.max_ep : nullptr;
+                            term_blk[(size_t)(cq - r0) * a.max_ep + e] =
+                                store_resolved<MODE>(A, flag, why, fe, we, A_rq, nullptr, e);
+                        };
+                        // MIXED queues longer than the block has threads: a lane per epoch, all by the general
+                        // solver. Populations that have gathered at a caustic queue thousands of epochs, so many
+                        // of them for the general solver that nearly every warp of six waits for one such lane,
+                        // where 32 lanes share its passes (152 curves of 500 epochs, 1024 x 300 generations:
+                        // 10.4 s, 12.4 s with six epochs per warp throughout); the short queues of the first
+                        // generations are bound by one epoch's latency, and the groups' is a tenth.
+                        // An overflowing MIXED queue is longer than any block (FP64's cannot overflow), so that which
+                        // epochs it held shows in no result: the others went to the general solver in place.
+                        if (MODE == SBLM_MIXED && n_q > blockDim.x)
+                            resolve_queue_lanes(sink.queue, n_q, threadIdx.x, blockDim.x, cand_of, data_of, store);
+                        else
+                            resolve_queue(sink.queue, n_q, threadIdx.x >> 5, blockDim.x >> 5, cand_of, data_of, store);
+                        __syncthreads();
+                        if (threadIdx.x == 0) s_qcount = 0;
+                        for (int base = r0; base < r1; base += per_pass) {
+                            const int cand = base + group;
+                            const double* row = term_blk + (size_t)(min(cand, r1 - 1) - r0) * a.max_ep;
+                            const double chi = term_row_sum(row, n_ep, g, G, cand < r1);
+                            if (g == 0 && cand < r1) s_chi[cand] = chi;
+                        }
+                        __syncthreads();
+                    }
                 }
                 if (a.blend) {  // Section 4.4: chi^2 of f A + (1 - f) with f profiled out, per candidate
                     for (int base = 0; base < n_pop; base += per_pass) {
@@ -590,11 +597,19 @@ sblm_status prepare(const double* t, const double* flux, const double* sigma, co
     SBLM_TRY(is_device_pointer(flux, &d2));
     SBLM_TRY(is_device_pointer(sigma, &d3));
     if (!d1 && !d2 && !d3) SBLM_TRY(check_lightcurve_host(t, flux, sigma, (int)total));
-    // per block: room for a quarter of a generation's epochs (a population gathered on a
+    // FP64: the block empties its queue after as many rows as hold 2^18 epochs (whole passes of the block's
+    // groups where it can), and the queue has room for all of them: 16 MB per block at most, whatever the
+    // population and the curve. 32 rows of the longest curves a block can stage still occupy every group.
+    const int per_pass = threads / G;
+    int rows = mode == SBLM_FP64 ? (int)std::max<long>(1, (1L << 18) / max_ep) : c.n_pop;
+    if (rows >= per_pass && rows < c.n_pop) rows -= rows % per_pass;
+    rows = std::min(rows, c.n_pop);
+    // MIXED, per block: room for a quarter of a generation's epochs (a population gathered on a
     // caustic-crossing model defers many), within 2^26 entries (~3 GB) over all blocks; when more defer,
     // all of them take the general solver, those past this in place, one divergent lane at a time
     const unsigned qcap =
-        mode != SBLM_FP32
+        mode == SBLM_FP64 ? (unsigned)rows * (unsigned)max_ep
+        : mode == SBLM_MIXED
             ? (unsigned)std::max<long>(4096, std::min<long>((long)c.n_pop * max_ep / 4, (1L << 26) / blocks))
             : 0;
     const int k_order = st.scratch(sizeof(int) * n_lc);
@@ -605,7 +620,7 @@ sblm_status prepare(const double* t, const double* flux, const double* sigma, co
     const int k_ie = st.scratch(n_isl > 1 ? sizeof(double) * SBLM_NPAR * (size_t)blocks * n_isl : 0);
     const int k_keys = st.scratch(sizeof(uint64_t) * (size_t)c.n_pop * SBLM_NPAR * blocks);
     const int k_q = st.scratch(deferred_entry_bytes() * (size_t)qcap * blocks);
-    const int k_term = st.scratch(mode != SBLM_FP32 ? sizeof(double) * (size_t)c.n_pop * max_ep * blocks : 0);
+    const int k_term = st.scratch(mode != SBLM_FP32 ? sizeof(double) * (size_t)rows * max_ep * blocks : 0);
     const int k_cand = st.scratch(sizeof(Cand) * (size_t)c.n_pop * blocks);
     const int k_next = st.scratch(sizeof(unsigned));
     const int k_genes = st.scratch(sizeof(double) * SBLM_NPAR * (size_t)n_lc);
@@ -684,6 +699,7 @@ sblm_status prepare(const double* t, const double* flux, const double* sigma, co
     a.keys = static_cast<uint64_t*>(st.scratch_ptr(k_keys));
     a.queue = static_cast<Deferred*>(st.scratch_ptr(k_q));
     a.qcap = qcap;
+    a.rows = rows;
     a.term = static_cast<double*>(st.scratch_ptr(k_term));
     a.cands = static_cast<Cand*>(st.scratch_ptr(k_cand));
     a.next = static_cast<unsigned*>(st.scratch_ptr(k_next));
