@@ -40,7 +40,7 @@ struct ForwardArgs {
     void* mixed = nullptr;
 };
 
-// MIXED and FP64 scratch of one forward pass: the re-solve queue (DeferSink in forward_run.cuh says what
+// MIXED and FP64 scratch of one forward pass: the re-solve queue (DeferSink in epochs.cuh says what
 // happens when it is full), its counter, the decoded candidates and, when chi^2 is wanted, the dense
 // n_cand x n_ep array of chi^2 terms that is summed row by row in a fixed order. FP64 passes its
 // candidates through one chunk's scratch (2^22 epochs: 0.25 GB). FP32 needs none (0 bytes).

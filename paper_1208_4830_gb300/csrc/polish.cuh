@@ -68,7 +68,7 @@ __device__ double block_chi2(const double* g, const Bounds& b, const LCView& vie
         if (threadIdx.x == 0) *sink.queue_count = 0;
         __syncthreads();
     }
-    double chi = eval_run<MODE, true, true>(k, true, 0, e0, e1, seg, view, A_row, nullptr, sink, term_row);
+    double chi = polish_epochs<MODE>(k, e0, e1, seg, view, A_row, sink, term_row);
     if constexpr (MODE == SBLM_MIXED) {
         __syncthreads();
         const unsigned n = min(*sink.queue_count, sink.queue_cap);

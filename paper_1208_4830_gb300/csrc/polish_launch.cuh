@@ -16,7 +16,7 @@ constexpr int kPolishMaxFev = 1 << 20;
 constexpr size_t kPolishSmemBudget = 200 * 1024;
 
 // MIXED scratch of one polish block: a re-solve queue with room for every epoch of the longest
-// lightcurve and its chi^2 term row (forward_run.cuh: DeferSink)
+// lightcurve and its chi^2 term row (epochs.cuh: DeferSink)
 struct PolishMixed {
     unsigned queue_cap = 0;
     size_t off_term = 0, block_bytes = 0;
