@@ -44,8 +44,11 @@ struct Refined {
     bool image;  // the corrections converged: a solution of the lens equation
 };
 
-// Newton steps on the lens equation from (z, w); at most `cap` corrections
-__device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<double> zeta, double q, int cap) {
+// Newton steps on the lens equation from (z, w); at most `cap` corrections. `short_first`: the residual of the
+// first correction to 2^-40 only, enough for an error of FP32's size at an image with |det J| above 0.1 (below 0.03
+// it would cost a third correction).
+__device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<double> zeta, double q, int cap,
+                                               bool short_first) {
     Refined o;
     o.image = false;
     o.det = 1.0;
@@ -54,9 +57,9 @@ __device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<do
 #pragma unroll 1
     for (int it = 0;; ++it) {
         const double n1 = norm2(z), n2 = norm2(w);
-        // the first correction is one of FP32's errors, and one Newton step gives its residual 2^-40
+        const bool full = it > 0 || !short_first;
         double r1 = rcp_start(n1), r2 = rcp_start(n2);
-        if (it > 0) {
+        if (full) {
             r1 = rcp_step(n1, r1);
             r2 = rcp_step(n2, r2);
         }
@@ -79,7 +82,7 @@ __device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<do
         const float n1f = (float)n1, n2f = (float)n2;
         const float scale = sqrt_(n1f) + sqrt_(r1f) + qf * sqrt_(r2f) + zeta_abs;
         const float lim = fmax(kRefineStep * fmin(ad, 1.f) * sqrt_(fmin(n1f, n2f)), 1e-15f * scale * rad);
-        const bool last = it > 0 && d2 <= lim * lim;
+        const bool last = full && d2 <= lim * lim;
         if (last) {
             // K in FP64 at (z, w), and det J advanced by delta: dK = 2 conj(delta) (q v^3 - u^3)
             const double uu = r1 * r1, vv = qr2 * r2;
@@ -133,7 +136,7 @@ __device__ __forceinline__ bool refine_images(const Root<float> rp[5], unsigned 
         cx<double> z, w;
         w = mk<double>(r.local ? (double)r.w.re : (double)r.z.re - d, r.local ? (double)r.w.im : (double)r.z.im);
         z = mk<double>(r.local ? d + w.re : (double)r.z.re, r.local ? w.im : (double)r.z.im);
-        const Refined f = refine_root(z, w, zeta, q, 4);
+        const Refined f = refine_root(z, w, zeta, q, 4, true);
         const cx<float> moved = mk<float>((float)(f.w.re - w.re), (float)(f.w.im - w.im));
         ok = ok && f.image && norm2(moved) <= 1e-6f * gap2;
         const double a = fabs(f.det);
@@ -313,7 +316,7 @@ __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<doubl
     f.z = z;
     f.w = w;
     f.det = 1.0;
-    if (open) f = refine_root(z, w, zeta, q, 8);
+    if (open) f = refine_root(z, w, zeta, q, 8, false);
     drop_duplicates(f, base, r);
     int count, parity;
     count_images(f, base, &count, &parity);
@@ -348,7 +351,7 @@ __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<doubl
         h.z = x;
         h.w = xw;
         h.det = 1.0;
-        if (mine) h = refine_root(x, xw, zeta, q, 6);
+        if (mine) h = refine_root(x, xw, zeta, q, 6, false);
         const cx<float> moved = mk<float>((float)(h.w.re - xw.re), (float)(h.w.im - xw.im));
         h.image = h.image && norm2(moved) <= 0.25f * gap2;
         const unsigned dups = drop_duplicates(h, base, r) >> base & 31u;
@@ -405,7 +408,7 @@ __device__ __forceinline__ bool resolve_thread(const cx<float>* z32, cx<double> 
     for (int i = 0; i < 5; ++i) {
         cx<double> z, w;
         start_from_fp32(z32[i], d, z, w);
-        const Refined f = refine_root(z, w, zeta, q, 8);
+        const Refined f = refine_root(z, w, zeta, q, 8, false);
         if (!f.image) continue;
         const cx<float> zf = mk<float>((float)f.z.re, (float)f.z.im), wf = mk<float>((float)f.w.re, (float)f.w.im);
         bool dup = false;
