@@ -48,7 +48,14 @@ typedef enum {
 
 /* Arithmetic of the forward model. */
 enum {
-    SBLM_FP64 = 0,  /* everything in FP64 */
+    SBLM_FP64 = 0,  /* FP64 magnifications: the quintic's roots in FP32 tell images from spurious
+                       roots, and every image is refined in FP64 on the lens equation. Epochs that
+                       FP32 may misjudge (wider triggers than MIXED's) are re-solved in FP64, as are
+                       lenses outside q in [5e-5, 30] or d in [0.25, 10] and sources beyond 64 or
+                       within 1e-6 of a lens: the ranges over which the refined results were compared
+                       with an FP64 solution of the quintic (20M epochs of caustic-crossing
+                       trajectories; relative 1e-10 where |det J| >= 1e-3). The amoeba solves every
+                       epoch's quintic in FP64. chi^2 in FP64 */
     SBLM_MIXED = 1, /* FP32 quintic solve; FP64 re-solve and polish of an epoch when triggered
                        (|det J| < 3e-2 at an image or at a rejected root that nearly solves
                        the lens equation, two roots closer than 1e-4, or an ambiguous image
@@ -146,7 +153,8 @@ void sblm_ea_params_default(sblm_ea_params* p);
  *                           an image (or a rejected root with a relative lens-equation residual
  *                           below 0.05) has |det J| < 3e-2, bit 5 = two images closer than 1e-4
  *                           (bits 4-5: FP32 and MIXED; in MIXED any of bits 0 and 2-5 of the FP32
- *                           solution triggers the FP64 re-solve, and they stay set beside bit 1)
+ *                           solution triggers the FP64 re-solve, and they stay set beside bit 1; FP64
+ *                           sets bits 0 and 2 only, at epochs left to the general FP64 solver)
  * n_cand >= 0, n_ep >= 0 (zero sizes return SBLM_OK without a launch). Host theta rows are checked
  * (finite, tE, d, q > 0); device rows are not, and an invalid row yields NaN or garbage in its
  * own outputs only.
@@ -157,11 +165,9 @@ sblm_status sblm_magnification(const double* theta, int32_t n_cand, const double
 /*
  * chi^2 of every candidate against one lightcurve (Section 4.1):
  * chi2_out[c] = sum_k ((flux_k - A_ck) / sigma_k)^2, A as in sblm_magnification, the model flux
- * of a unit, unblended source. The sum runs in FP64-grade arithmetic in every precision (FP32
- * modes accumulate each thread's epochs as a float pair) and in a fixed order, so FP64 and FP32
- * results are deterministic; in MIXED the terms of the epochs re-solved in FP64 are added
- * atomically, so the last bits of a MIXED chi^2 can vary from run to run. sigma_k > 0 and finite data are required: host buffers are checked
- * (SBLM_EINVAL); device buffers are not read back for a check, and bad data there turn into
+ * of a unit, unblended source. The sum runs in FP64 and in a fixed order, so equal calls return
+ * the same bits in every precision. sigma_k > 0 and finite data are required: host buffers are
+ * checked (SBLM_EINVAL); device buffers are not read back for a check, and bad data there turn into
  * non-finite chi^2 values (which the EA ranks last). n_ep == 0 gives chi^2 = 0.
  */
 sblm_status sblm_chi2(const double* theta, int32_t n_cand, const double* t, const double* flux,

@@ -314,11 +314,12 @@ __global__ void __launch_bounds__(kBatchMaxThreads, 1) batch_fit_kernel(BatchArg
                                 store_resolved<MODE>(A, flag, why, fe, we, A_rq, nullptr, e);
                         };
                         // MIXED queues longer than the block has threads: a lane per epoch, all by the general
-                        // solver. Populations that have gathered at a caustic queue thousands of epochs, so many
-                        // of them for the general solver that nearly every warp of six waits for one such lane,
-                        // where 32 lanes share its passes (152 curves of 500 epochs, 1024 x 300 generations:
-                        // 10.4 s, 12.4 s with six epochs per warp throughout); the short queues of the first
-                        // generations are bound by one epoch's latency, and the groups' is a tenth.
+                        // solver. 152 curves of 500 epochs, 1024 rows: 300 generations 10.4 s, 12.3 s with the
+                        // groups throughout (60 generations 2.05 and 2.56 s). The slowest curve sets these: its
+                        // population has gathered at a caustic and queues 20,000 epochs a generation, 9% of which need
+                        // the groups' second stage (resolve_group: FP64 roots), so that a third of its warps of six
+                        // wait for it. The short queues of the first generations are bound by one epoch's latency,
+                        // and the groups' is a tenth.
                         // An overflowing MIXED queue is longer than any block (FP64's cannot overflow), so that which
                         // epochs it held shows in no result: the others went to the general solver in place.
                         if (MODE == SBLM_MIXED && n_q > blockDim.x)

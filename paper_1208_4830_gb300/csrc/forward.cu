@@ -29,7 +29,7 @@ constexpr int kResolveBlock = 128;
 // MIXED and FP64, second pass: the queued epochs, six per warp (refine.cuh), over the whole GPU: the
 // first epochs of the queue go to one warp of every block, so that a short queue spreads over the SMs
 // (the FP64 pipe is the bound; 131,072 x 2000: 10.1 ms with one lane per epoch and the general solver,
-// 5.9 ms so; 1000 x 100: 370 us, 63 us). Each chi^2 term goes to its (candidate, epoch) place in
+// 6.1 ms so; 1000 x 100: 370 us, 63 us). Each chi^2 term goes to its (candidate, epoch) place in
 // the dense term array (no atomics), so the sums of the third pass do not depend on the order in which
 // the queue was filled.
 template <int MODE, bool CHI2>
