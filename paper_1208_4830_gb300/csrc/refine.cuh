@@ -44,57 +44,74 @@ struct Refined {
     bool image;  // the corrections converged: a solution of the lens equation
 };
 
-// Newton steps on the lens equation from (z, w); at most `cap` corrections. `short_first`: the residual of the
+// One Newton step on the lens equation at (z, w), r1 and r2 the reciprocals of norm2(z) and norm2(w): the FP64
+// residual's correction by the FP32 Jacobian, and the FP32 terms it was taken from
+struct LensStep {
+    cx<float> delta, u, v, K;
+    float dj_abs, dj_rcp;
+};
+__device__ __forceinline__ LensStep lens_step(cx<double> z, cx<double> w, double r1, double r2, cx<double> zeta, double q) {
+    LensStep o;
+    const double qr2 = q * r2;
+    // u = 1/conj(z) = z r1, v = 1/(d - conj(z)) = -w r2; f = z - u + q v - zeta
+    cx<double> f;
+    f.re = fma(-w.re, qr2, fma(-z.re, r1, z.re)) - zeta.re;
+    f.im = fma(-w.im, qr2, fma(-z.im, r1, z.im)) - zeta.im;
+    const float qf = (float)q, r1f = (float)r1, r2f = (float)r2;
+    const cx<float> zf = mk<float>((float)z.re, (float)z.im), wf = mk<float>((float)w.re, (float)w.im);
+    const cx<float> ff = mk<float>((float)f.re, (float)f.im);
+    o.u = r1f * zf;
+    o.v = (-r2f) * wf;
+    o.K = o.u * o.u + qf * (o.v * o.v);
+    const float dj = 1.f - norm2(o.K);
+    o.dj_abs = fabs(dj);
+    const cx<float> num = o.K * conj(ff) - ff;
+    o.dj_rcp = rcp(o.dj_abs);
+    o.delta = (dj < 0.f ? -o.dj_rcp : o.dj_rcp) * num;
+    return o;
+}
+
+// Newton steps on the lens equation from (z, w); at most `cap` corrections. SHORT_FIRST: the residual of the
 // first correction to 2^-40 only, enough for an error of FP32's size at an image with |det J| above 0.1 (below 0.03
 // it would cost a third correction).
-__device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<double> zeta, double q, int cap,
-                                               bool short_first) {
+template <bool SHORT_FIRST>
+__device__ __forceinline__ Refined refine_root(cx<double> z, cx<double> w, cx<double> zeta, double q, int cap) {
     Refined o;
     o.image = false;
     o.det = 1.0;
+    if (SHORT_FIRST) {
+        const cx<float> delta = lens_step(z, w, rcp_start(norm2(z)), rcp_start(norm2(w)), zeta, q).delta;
+        z = mk<double>(z.re + (double)delta.re, z.im + (double)delta.im);
+        w = mk<double>(w.re + (double)delta.re, w.im + (double)delta.im);
+        --cap;
+    }
     const float qf = (float)q;
     const float zeta_abs = sqrt_(norm2(mk<float>((float)zeta.re, (float)zeta.im)));
 #pragma unroll 1
     for (int it = 0;; ++it) {
         const double n1 = norm2(z), n2 = norm2(w);
-        const bool full = it > 0 || !short_first;
-        double r1 = rcp_start(n1), r2 = rcp_start(n2);
-        if (full) {
-            r1 = rcp_step(n1, r1);
-            r2 = rcp_step(n2, r2);
-        }
-        const double qr2 = q * r2;
-        // u = 1/conj(z) = z r1, v = 1/(d - conj(z)) = -w r2; f = z - u + q v - zeta
-        cx<double> f;
-        f.re = fma(-w.re, qr2, fma(-z.re, r1, z.re)) - zeta.re;
-        f.im = fma(-w.im, qr2, fma(-z.im, r1, z.im)) - zeta.im;
-        const float r1f = (float)r1, r2f = (float)r2;
-        const cx<float> zf = mk<float>((float)z.re, (float)z.im), wf = mk<float>((float)w.re, (float)w.im);
-        const cx<float> u = r1f * zf, v = (-r2f) * wf, ff = mk<float>((float)f.re, (float)f.im);
-        const cx<float> K = u * u + qf * (v * v);
-        const float dj = 1.f - norm2(K), ad = fabs(dj);
-        const cx<float> num = K * conj(ff) - ff;
-        const float rad = rcp(ad);
-        const cx<float> delta = (dj < 0.f ? -rad : rad) * num;
-        const float d2 = norm2(delta);
+        const double r1 = rcp_normal(n1), r2 = rcp_normal(n2);
+        const LensStep s = lens_step(z, w, r1, r2, zeta, q);
+        const float d2 = norm2(s.delta);
         if (!isfinite(d2)) break;
         // stop at the step bound, or at the rounding level of f's FP64 evaluation
         const float n1f = (float)n1, n2f = (float)n2;
-        const float scale = sqrt_(n1f) + sqrt_(r1f) + qf * sqrt_(r2f) + zeta_abs;
-        const float lim = fmax(kRefineStep * fmin(ad, 1.f) * sqrt_(fmin(n1f, n2f)), 1e-15f * scale * rad);
-        const bool last = full && d2 <= lim * lim;
+        const float scale = sqrt_(n1f) + sqrt_((float)r1) + qf * sqrt_((float)r2) + zeta_abs;
+        const float lim =
+            fmax(kRefineStep * fmin(s.dj_abs, 1.f) * sqrt_(fmin(n1f, n2f)), 1e-15f * scale * s.dj_rcp);
+        const bool last = d2 <= lim * lim;
         if (last) {
             // K in FP64 at (z, w), and det J advanced by delta: dK = 2 conj(delta) (q v^3 - u^3)
-            const double uu = r1 * r1, vv = qr2 * r2;
+            const double uu = r1 * r1, vv = q * r2 * r2;
             const double kr = fma(fma(z.re, z.re, -(z.im * z.im)), uu, fma(w.re, w.re, -(w.im * w.im)) * vv);
             const double ki = fma(z.re * z.im, uu, (w.re * w.im) * vv);
-            const cx<float> dK = (2.f * conj(delta)) * (qf * (v * v * v) - u * u * u);
-            const float ddet = -2.f * (K.re * dK.re + K.im * dK.im);
+            const cx<float> dK = (2.f * conj(s.delta)) * (qf * (s.v * s.v * s.v) - s.u * s.u * s.u);
+            const float ddet = -2.f * (s.K.re * dK.re + s.K.im * dK.im);
             o.det = fma(-4.0 * ki, ki, fma(-kr, kr, 1.0)) + (double)ddet;
             o.image = true;
         }
         if (!last && it >= cap) break;
-        const double dr = (double)delta.re, di = (double)delta.im;
+        const double dr = (double)s.delta.re, di = (double)s.delta.im;
         z = mk<double>(z.re + dr, z.im + di);
         w = mk<double>(w.re + dr, w.im + di);
         if (last) break;
@@ -136,7 +153,7 @@ __device__ __forceinline__ bool refine_images(const Root<float> rp[5], unsigned 
         cx<double> z, w;
         w = mk<double>(r.local ? (double)r.w.re : (double)r.z.re - d, r.local ? (double)r.w.im : (double)r.z.im);
         z = mk<double>(r.local ? d + w.re : (double)r.z.re, r.local ? w.im : (double)r.z.im);
-        const Refined f = refine_root(z, w, zeta, q, 4, true);
+        const Refined f = refine_root<true>(z, w, zeta, q, 4);
         const cx<float> moved = mk<float>((float)(f.w.re - w.re), (float)(f.w.im - w.im));
         ok = ok && f.image && norm2(moved) <= 1e-6f * gap2;
         const double a = fabs(f.det);
@@ -316,7 +333,7 @@ __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<doubl
     f.z = z;
     f.w = w;
     f.det = 1.0;
-    if (open) f = refine_root(z, w, zeta, q, 8, false);
+    if (open) f = refine_root<false>(z, w, zeta, q, 8);
     drop_duplicates(f, base, r);
     int count, parity;
     count_images(f, base, &count, &parity);
@@ -351,7 +368,7 @@ __device__ __forceinline__ bool resolve_group(cx<float> zf, bool valid, cx<doubl
         h.z = x;
         h.w = xw;
         h.det = 1.0;
-        if (mine) h = refine_root(x, xw, zeta, q, 6, false);
+        if (mine) h = refine_root<false>(x, xw, zeta, q, 6);
         const cx<float> moved = mk<float>((float)(h.w.re - xw.re), (float)(h.w.im - xw.im));
         h.image = h.image && norm2(moved) <= 0.25f * gap2;
         const unsigned dups = drop_duplicates(h, base, r) >> base & 31u;
@@ -408,7 +425,7 @@ __device__ __forceinline__ bool resolve_thread(const cx<float>* z32, cx<double> 
     for (int i = 0; i < 5; ++i) {
         cx<double> z, w;
         start_from_fp32(z32[i], d, z, w);
-        const Refined f = refine_root(z, w, zeta, q, 8, false);
+        const Refined f = refine_root<false>(z, w, zeta, q, 8);
         if (!f.image) continue;
         const cx<float> zf = mk<float>((float)f.z.re, (float)f.z.im), wf = mk<float>((float)f.w.re, (float)f.w.im);
         bool dup = false;
