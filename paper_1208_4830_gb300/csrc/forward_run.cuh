@@ -55,7 +55,7 @@ __device__ __forceinline__ double store_resolved(double A, uint8_t flag, uint32_
 // the general solver when the warp's lanes are nearly all taken, and at the end: FP64 instructions cost the same
 // for one lane as for 32, and lenses outside the refined range leave every epoch open. MIXED chi^2 of 4096 x
 // 2000 at q < 5e-5, d > 10, d < 0.25: 4.24, 4.75, 15.7 ms with the solver in place on the lanes r = 0, 2.97, 2.66,
-// 8.95 ms so; an FP64 batch at q < 1e-4 (152 curves, 128 x 6 generations): 635, 371 ms. `cand(c)` is candidate c, `data(c, e)` the epoch's time, flux and
+// 9.0 to 9.5 ms so; an FP64 batch at q < 1e-4 (152 curves, 128 x 6 generations): 635, 371 ms. `cand(c)` is candidate c, `data(c, e)` the epoch's time, flux and
 // 1/sigma, and `store(c, e, A, flag, why, fe, we)` takes the result (one lane per epoch). Every lane
 // of the warp calls it.
 struct EpochData {

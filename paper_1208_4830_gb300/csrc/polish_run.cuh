@@ -2,8 +2,8 @@
 // An epoch loop apart from forward_run.cuh's: the compiler fuses the FP32 products here in
 // another way at each of the kernel's call sites, and any change of the loop moves MIXED chi^2 by 1e-7,
 // which a simplex amplifies. What bounds the amoeba is the chain of one chi^2 after the other; the FP64
-// re-solves, each by one thread, were a third of it: 64 curves of 500 epochs, 200 evaluations, 29.1 ms with the
-// general solver for each, 24.7 ms with the epoch's roots refined first (resolve_thread). FP64 solves the
+// re-solves, each by one thread, were a third of it: 64 curves of 500 epochs, 200 evaluations, 32.0 ms with the
+// general solver for each, 25.1 ms with the epoch's roots refined first (resolve_thread). FP64 solves the
 // quintic of every epoch in FP64, warm from the previous epoch.
 #pragma once
 

@@ -12,7 +12,7 @@
 // Jacobian at the last point in FP64, advanced by that last correction to first order, gives det J.
 // 16 FP64 instructions for the first step, 20 for each further one and about 20 for the last one's Jacobian,
 // against some 250 per root and sweep of a root iteration in FP64. FP64 chi^2 of 4096 x 2000: 68.6 ms with the
-// quintic solved in FP64, 8.4 ms so; one event's curve of 400 epochs: 1186 us, 215 us.
+// quintic solved in FP64, 8.4 ms so; one event's curve of 400 epochs: 1129 us, 189 us.
 #pragma once
 
 #include "forward.cuh"
